@@ -14,12 +14,19 @@
 // Convolutions run on the tensor cores (unet_tc.cuh: implicit GEMM with
 // mma.sync, BF16 operands, FP32 accumulation; activations and output
 // gradients are staged channel-last with the channel count padded to a
-// multiple of 8).  The data gradient is the forward kernel on the output
-// gradient (rounded to BF16) with flipped, transposed weights; the weight
-// gradient reduces per-CTA partials in a fixed order (no atomics), so a
-// gradient is bit-reproducible.  Pooling/upsampling and their adjoints, the
-// normalised squared-error loss and Adam are plain elementwise kernels.
+// multiple of 8).  The upsampling and concatenation of the decoder are part
+// of the staging of its convolutions (and of their weight gradients), the
+// ReLU masks of the backward pass part of the epilogues that write the BF16
+// gradients.  As kernels of their own these passes took longer than the
+// convolutions: one thread per element with 64-bit divisions, 407 us to write
+// the 24-channel concatenation of 128^3 voxels.  The data gradient is the
+// forward kernel on the output gradient (rounded to BF16) with flipped,
+// transposed weights; the weight gradient reduces per-CTA partials in a fixed
+// order (no atomics), so a gradient is bit-reproducible.  Pooling, the
+// adjoints that join two paths, the normalised squared-error loss and Adam
+// are elementwise kernels, eight channels (16 bytes) per thread.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -36,131 +43,211 @@ struct Shape { int B, D, H, W; };
 __host__ __device__ inline int64_t vox(const Shape& s) { return (int64_t)s.B * s.D * s.H * s.W; }
 
 
-// 2x average pooling (and its adjoint: nearest up-spread divided by 2^d)
-__global__ void k_pool(const __nv_bfloat16* X, Shape s, int c, int pz, __nv_bfloat16* Y) {
-    Shape o{s.B, pz ? s.D / 2 : s.D, s.H / 2, s.W / 2};
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= vox(o) * c) return;
-    int ch = e % c;
-    int64_t v = e / c;
-    int x = v % o.W, y = (v / o.W) % o.H, z = (v / ((int64_t)o.W * o.H)) % o.D, b = v / ((int64_t)o.W * o.H * o.D);
-    float sum = 0.f;
-    int nz = pz ? 2 : 1;
-    for (int dz = 0; dz < nz; ++dz)
+__device__ __forceinline__ void unpack8(const uint4& w, float (&f)[8]) {
+    const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        f[2 * k] = __uint_as_float(u[k] << 16);
+        f[2 * k + 1] = __uint_as_float(u[k] & 0xffff0000u);
+    }
+}
+__device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
+    uint32_t u[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * k], f[2 * k + 1]);
+        u[k] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    return make_uint4(u[0], u[1], u[2], u[3]);
+}
+__device__ __forceinline__ void load8(const float* p, float (&f)[8]) {
+    const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+    f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w;
+    f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+}
+// item e of (voxel, group of 8 channels) -> coordinates
+struct Item { int b, z, y, x, k; };
+__device__ __forceinline__ Item item_of(int64_t e, const Shape& s, int ng) {
+    Item i;
+    const uint32_t v = (uint32_t)(e / ng);                // fewer than 2^31 voxels per level in any buffer that fits
+    i.k = (int)(e - (int64_t)v * ng);
+    uint32_t r = v / (uint32_t)s.W;
+    i.x = (int)(v - r * (uint32_t)s.W);
+    uint32_t q = r / (uint32_t)s.H;
+    i.y = (int)(r - q * (uint32_t)s.H);
+    i.b = (int)(q / (uint32_t)s.D);
+    i.z = (int)(q - (uint32_t)i.b * (uint32_t)s.D);
+    return i;
+}
+__device__ __forceinline__ int64_t vox_at(const Shape& s, int b, int z, int y, int x) {
+    return (((int64_t)b * s.D + z) * s.H + y) * s.W + x;
+}
+
+// 2x average pooling: X fine (shape s), Y coarse (shape o); c a multiple of 8
+__global__ void __launch_bounds__(256) k_pool(const __nv_bfloat16* __restrict__ X, Shape s, Shape o, int c, int pz,
+                                              __nv_bfloat16* __restrict__ Y) {
+    const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (e >= vox(o) * (c / 8)) return;
+    const Item i = item_of(e, o, c / 8);
+    float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int dz = 0; dz < 1 + pz; ++dz)
+#pragma unroll
         for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
             for (int dx = 0; dx < 2; ++dx) {
-                int zz = pz ? 2 * z + dz : z;
-                sum += __bfloat162float(X[((((int64_t)b * s.D + zz) * s.H + 2 * y + dy) * s.W + 2 * x + dx) * c + ch]);
+                float f[8];
+                unpack8(*reinterpret_cast<const uint4*>(
+                            X + vox_at(s, i.b, pz ? 2 * i.z + dz : i.z, 2 * i.y + dy, 2 * i.x + dx) * c + 8 * i.k), f);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) sum[k] += f[k];
             }
-    Y[e] = __float2bfloat16(sum / (nz * 4));
+    const float inv = pz ? 0.125f : 0.25f;                // exact
+#pragma unroll
+    for (int k = 0; k < 8; ++k) sum[k] *= inv;
+    *reinterpret_cast<uint4*>(Y + e * 8) = pack8(sum);
 }
 
-__global__ void k_pool_adj(const float* dY, Shape s, int c, int pz, float* dX) {  // s: fine shape
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= vox(s) * c) return;
-    int ch = e % c;
-    int64_t v = e / c;
-    int x = v % s.W, y = (v / s.W) % s.H, z = (v / ((int64_t)s.W * s.H)) % s.D, b = v / ((int64_t)s.W * s.H * s.D);
-    Shape o{s.B, pz ? s.D / 2 : s.D, s.H / 2, s.W / 2};
-    int zc = pz ? z / 2 : z;
-    dX[e] += dY[((((int64_t)b * o.D + zc) * o.H + y / 2) * o.W + x / 2) * c + ch] / ((pz ? 2 : 1) * 4);
+// Gradient at a decoder input's coarse part: the adjoint of the upsampling
+// (sum over the 2^d children of channels [0, c) of dY, fine, cy channels),
+// through the ReLU of the coarse activations act, rounded to BF16.
+__global__ void __launch_bounds__(256) k_up_adj(const float* __restrict__ dY, Shape s, Shape o, int c, int cy, int pz,
+                                                const __nv_bfloat16* __restrict__ act, __nv_bfloat16* __restrict__ g) {
+    const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (e >= vox(o) * (c / 8)) return;
+    const Item i = item_of(e, o, c / 8);
+    float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int dz = 0; dz < 1 + pz; ++dz)
+#pragma unroll
+        for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+            for (int dx = 0; dx < 2; ++dx) {
+                float f[8];
+                load8(dY + vox_at(s, i.b, pz ? 2 * i.z + dz : i.z, 2 * i.y + dy, 2 * i.x + dx) * cy + 8 * i.k, f);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) sum[k] += f[k];
+            }
+    float a[8];
+    unpack8(*reinterpret_cast<const uint4*>(act + e * 8), a);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) sum[k] = a[k] > 0.f ? sum[k] : 0.f;
+    *reinterpret_cast<uint4*>(g + e * 8) = pack8(sum);
 }
 
-// nearest 2x upsampling of X (coarse) into channels [0, c) of Y (fine, cy channels)
-__global__ void k_up_concat(const __nv_bfloat16* Xc, const __nv_bfloat16* skip, Shape s, int c, int cs, int pz,
-                            __nv_bfloat16* Y) {
-    int cy = c + cs;
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= vox(s) * cy) return;
-    int ch = e % cy;
-    int64_t v = e / cy;
-    if (ch < c) {
-        int x = v % s.W, y = (v / s.W) % s.H, z = (v / ((int64_t)s.W * s.H)) % s.D, b = v / ((int64_t)s.W * s.H * s.D);
-        Shape o{s.B, pz ? s.D / 2 : s.D, s.H / 2, s.W / 2};
-        int zc = pz ? z / 2 : z;
-        Y[e] = Xc[((((int64_t)b * o.D + zc) * o.H + y / 2) * o.W + x / 2) * c + ch];
-    } else {
-        Y[e] = skip[v * cs + (ch - c)];
-    }
-}
-
-// adjoint of k_up_concat: coarse gradient (sum over the 2^d children) and
-// skip gradient (added)
-__global__ void k_up_concat_adj(const float* dY, Shape s, int c, int cs, int pz, float* dXc, float* dskip) {
-    int cy = c + cs;
-    Shape o{s.B, pz ? s.D / 2 : s.D, s.H / 2, s.W / 2};
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t nco = vox(o) * c, nsk = vox(s) * cs;
-    if (e < nco) {
-        int ch = e % c;
-        int64_t v = e / c;
-        int x = v % o.W, y = (v / o.W) % o.H, z = (v / ((int64_t)o.W * o.H)) % o.D, b = v / ((int64_t)o.W * o.H * o.D);
-        float sum = 0.f;
-        int nz = pz ? 2 : 1;
-        for (int dz = 0; dz < nz; ++dz)
-            for (int dy = 0; dy < 2; ++dy)
-                for (int dx = 0; dx < 2; ++dx) {
-                    int zz = pz ? 2 * z + dz : z;
-                    sum += dY[((((int64_t)b * s.D + zz) * s.H + 2 * y + dy) * s.W + 2 * x + dx) * cy + ch];
-                }
-        dXc[e] = sum;
-    }
-    if (e < nsk) {
-        int ch = e % cs;
-        int64_t v = e / cs;
-        dskip[e] += dY[v * cy + c + ch];
-    }
-}
-
-// gradient through ReLU: g *= (y > 0); g may be FP32 accumulated from several paths
-__global__ void k_relu_bwd(float* g, const __nv_bfloat16* y, int64_t n) {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < n && !(__bfloat162float(y[e]) > 0.f)) g[e] = 0.f;
+// Gradient at an encoder level's output, which feeds the skip connection
+// (channels [c0, c0 + c) of dY, cy channels) and the pooling (its gradient dP,
+// coarse): their sum through the ReLU of act, rounded to BF16.
+__global__ void __launch_bounds__(256) k_skip_pool_adj(const float* __restrict__ dY, const float* __restrict__ dP,
+                                                       Shape s, Shape o, int c, int c0, int cy, int pz,
+                                                       const __nv_bfloat16* __restrict__ act,
+                                                       __nv_bfloat16* __restrict__ g) {
+    const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    const int ng = c / 8;
+    if (e >= vox(s) * ng) return;
+    const Item i = item_of(e, s, ng);
+    float f[8], p[8], a[8];
+    load8(dY + (e / ng) * cy + c0 + 8 * i.k, f);
+    load8(dP + vox_at(o, i.b, pz ? i.z / 2 : i.z, i.y / 2, i.x / 2) * c + 8 * i.k, p);
+    unpack8(*reinterpret_cast<const uint4*>(act + e * 8), a);
+    const float inv = pz ? 0.125f : 0.25f;                // exact
+#pragma unroll
+    for (int k = 0; k < 8; ++k) f[k] = a[k] > 0.f ? f[k] + p[k] * inv : 0.f;
+    *reinterpret_cast<uint4*>(g + e * 8) = pack8(f);
 }
 
 // loss = mean_b ||out_b - y_b||^2 / ||y_b||^2; g = d loss / d out.  The two
 // sums per sample are reduced deterministically: per-block partials (warp
-// shuffles, then warps in order), then the blocks in order.
-constexpr int LOSS_BLOCKS = 64;
-__global__ void k_loss_partials(const float* out, const float* y, int64_t per, double* part) {
+// shuffles, then warps in order), then the blocks in order.  FP64 arithmetic
+// and conversions are slow on this part (two per clock and SM): the squares
+// are summed as float-float pairs (TwoProd, TwoSum: about 2^-44 relative) and
+// the gradient's factor 2 / (||y||^2 B) is kept as a float-float pair, its
+// product with out - y then accurate to about 2^-47 before it is rounded
+// (with an FP64 division per element: 319 us for 8.4 M elements).
+constexpr int LOSS_BLOCKS = 256;      // most blocks per sample
+struct SumFF {
+    float hi = 0.f, lo = 0.f;
+    __device__ void square(float a) {
+        const float p = a * a, e = fmaf(a, a, -p);
+        float s, t;
+        stk::two_sum(hi, p, s, t);
+        lo += t + e;
+        hi = s;
+    }
+    __device__ double warp() const { return stk::warp_sum_ff(hi, lo); }
+};
+__global__ void __launch_bounds__(256) k_loss_partials(const float* __restrict__ out, const float* __restrict__ y,
+                                                       int64_t per, double* part) {
     __shared__ double red[2][8];
     const int b = blockIdx.y;
-    double num = 0.0, den = 0.0;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < per; e += (int64_t)gridDim.x * blockDim.x) {
-        float d = out[b * per + e] - y[b * per + e];
-        num += (double)d * d;
-        den += (double)y[b * per + e] * y[b * per + e];
+    SumFF num, den;
+    const float* ob = out + b * per;
+    const float* yb = y + b * per;
+    const int64_t step = (int64_t)gridDim.x * 256;
+    int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    for (; e + 3 * step < per; e += 4 * step) {
+        float o[4], t[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { o[k] = ob[e + k * step]; t[k] = yb[e + k * step]; }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { num.square(o[k] - t[k]); den.square(t[k]); }
     }
-    num = warp_sum(num);
-    den = warp_sum(den);
+    for (; e < per; e += step) { const float t = yb[e]; num.square(ob[e] - t); den.square(t); }
+    const double dn = num.warp(), dd = den.warp();
     const int w = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) { red[0][w] = num; red[1][w] = den; }
+    if ((threadIdx.x & 31) == 0) { red[0][w] = dn; red[1][w] = dd; }
     __syncthreads();
     if (threadIdx.x == 0) {
         double a = 0.0, c = 0.0;
-        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) { a += red[0][q]; c += red[1][q]; }
-        part[2 * (b * LOSS_BLOCKS + blockIdx.x)] = a;
-        part[2 * (b * LOSS_BLOCKS + blockIdx.x) + 1] = c;
+        for (int q = 0; q < 8; ++q) { a += red[0][q]; c += red[1][q]; }
+        part[2 * (b * gridDim.x + blockIdx.x)] = a;
+        part[2 * (b * gridDim.x + blockIdx.x) + 1] = c;
     }
 }
 
-__global__ void k_loss_finish(const double* part, int B, double* sums) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
+// One warp per sample: the blocks' partials, a fixed tree; then the
+// gradient's factor 2 / (||y||^2 B) = (f.x + f.y) 2^f.z (scaled by a power of
+// two, since it can lie outside the FP32 range), 0 for a sample whose target
+// is zero.
+__global__ void k_loss_finish(const double* part, int nblocks, int B, double* sums, float4* fac) {
+    const int b = blockIdx.x, lane = threadIdx.x;
     double a = 0.0, c = 0.0;
-    for (int q = 0; q < LOSS_BLOCKS; ++q) { a += part[2 * (b * LOSS_BLOCKS + q)]; c += part[2 * (b * LOSS_BLOCKS + q) + 1]; }
+    for (int q = lane; q < nblocks; q += 32) { a += part[2 * (b * nblocks + q)]; c += part[2 * (b * nblocks + q) + 1]; }
+    a = warp_sum(a);
+    c = warp_sum(c);
+    if (lane != 0) return;
     sums[2 * b] = a;
     sums[2 * b + 1] = c;
+    int ex = 0;
+    const double m = c > 0.0 ? frexp(2.0 / c / B, &ex) : 0.0;
+    const float fh = (float)m;
+    fac[b] = make_float4(fh, (float)(m - (double)fh), (float)ex, 0.f);
 }
 
-__global__ void k_loss_grad(const float* out, const float* y, int64_t per, int B, const double* sums, float* g) {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= per * B) return;
-    int b = e / per;
-    // a sample whose target is zero contributes nothing (no gradient)
-    if (!(sums[2 * b + 1] > 0.0)) { g[e] = 0.f; return; }
-    double den = sums[2 * b + 1];
-    g[e] = (float)(2.0 * (out[e] - y[e]) / den / B);
+// gradient of the loss at the output, in BF16 with cp channels (zero padded),
+// as the output convolution's backward kernels read it: four channels a thread
+__global__ void __launch_bounds__(256) k_loss_grad(const float* __restrict__ out, const float* __restrict__ y,
+                                                   int64_t nvox, int c, int cp, const float4* __restrict__ fac,
+                                                   __nv_bfloat16* __restrict__ g) {
+    const int nq = cp >> 2, per = 256 / nq;               // nq = 2 or 4
+    const int q = threadIdx.x & (nq - 1);
+    const int64_t vs = (int64_t)blockIdx.x * per + threadIdx.x / nq;
+    if (vs >= nvox) return;
+    const int64_t v = (int64_t)blockIdx.y * nvox + vs;
+    const float4 f = fac[blockIdx.y];
+    const int ex = (int)f.z;
+    float r[4] = {0.f, 0.f, 0.f, 0.f};
+    if (4 * q < c && f.x != 0.f) {
+        const float* po = out + v * c + 4 * q;
+        const float* py = y + v * c + 4 * q;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float d = po[k] - py[k];
+            const float p = d * f.x;
+            r[k] = ldexpf(isfinite(p) ? p + (fmaf(d, f.x, -p) + d * f.y) : p, ex);
+        }
+    }
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(r[0], r[1]), hi = __floats2bfloat162_rn(r[2], r[3]);
+    *reinterpret_cast<uint2*>(g + v * cp + 4 * q) =
+        make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
 }
 
 __global__ void k_adam(float* th, const float* g, float* m, float* v, int64_t n, float lr, float b1, float b2,
@@ -196,17 +283,20 @@ struct stokes_net_s {
     // every change of the parameters
     std::vector<__nv_bfloat16*> wf, wg;
     bool wf_valid = false;
-    __nv_bfloat16* g16 = nullptr;   // output gradient of the layer in BF16 (cp(cout) channels)
+    __nv_bfloat16 *gA = nullptr, *gB = nullptr;   // output gradients of two consecutive layers in BF16
     float* part = nullptr;          // weight-gradient partials, part_ctas x part_stride floats
-    int part_ctas = 0, sms = 0;
+    int part_ctas = 0, sms = 0, device = 0;
     int adam_t = 0;
     // activations (BF16) and gradients (FP32)
     __nv_bfloat16 *xin = nullptr, *e0a = nullptr, *e0 = nullptr, *p0 = nullptr, *e1a = nullptr, *e1 = nullptr,
-                  *p1 = nullptr, *e2a = nullptr, *e2 = nullptr, *c1 = nullptr, *d1a = nullptr, *d1 = nullptr,
-                  *c0 = nullptr, *d0a = nullptr, *d0 = nullptr;
+                  *p1 = nullptr, *e2a = nullptr, *e2 = nullptr, *d1a = nullptr, *d1 = nullptr, *d0a = nullptr,
+                  *d0 = nullptr;
     float* out = nullptr;
-    float *g_a = nullptr, *g_b = nullptr, *g_skip0 = nullptr, *g_skip1 = nullptr, *g_c = nullptr;
+    // FP32 data gradients at the decoder inputs (24 and 48 channels) and at
+    // the pooled tensors (8 and 16 channels)
+    float *g_c0 = nullptr, *g_c1 = nullptr, *g_p0 = nullptr, *g_p1 = nullptr;
     double* sums = nullptr;
+    float4* fac = nullptr;          // per sample: the loss gradient's factor
     std::vector<void*> allocs;
     cudaStream_t s = nullptr;
     std::string err;
@@ -218,33 +308,58 @@ using unet_tc::cp8;
 // (cin, cout) the network supports: the tensor-core kernels are instantiated
 // for input channels padded to 8 or 16 and output channels padded to 8 or 16
 bool io_channels_ok(int c) { return c == 4 || c == 8 || c == 12 || c == 16; }
+constexpr int MAX_DEVICES = 64;
 constexpr int PART_STRIDE = 27 * 32 * 32 + 32;     // largest taps x cp(cin) x cp(cout) + cp(cout)
 
 int taps_of(const stokes_net_s* n, const Conv& c) { return (n->KZ == 3 && c.ks == 3 ? 3 : 1) * c.ks * c.ks; }
 
-template <int KZ, int KS, int CP, int COUTP>
-cudaError_t launch_conv_tc(stokes_net_s* n, const __nv_bfloat16* X, Shape s, const __nv_bfloat16* Wp,
-                           const float* bias, int cout, int relu, __nv_bfloat16* Yb, float* Yf) {
+// CTAs of a persistent kernel: the tiles, at most what fits on the device
+// (and `cap`); resident: the kernel's cached answer for this process.
+template <class K>
+int persistent_ctas(const stokes_net_s* n, K k, size_t smem, int tiles, int cap, std::atomic<int>& resident) {
+    int per = resident.load(std::memory_order_relaxed);
+    if (per <= 0) {
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 256, smem);
+        per = std::max(per, 1);
+        resident.store(per, std::memory_order_relaxed);
+    }
+    return std::max(1, std::min({tiles, std::max(n->sms, 1) * per, cap}));
+}
+
+// Operands of one convolution: input (X, and Xc for the upsampled channels),
+// packed weights, epilogue.
+struct ConvArgs {
+    const __nv_bfloat16 *X = nullptr, *Xc = nullptr, *Wp = nullptr, *mask = nullptr;
+    const float* bias = nullptr;
+    int cout = 0, relu = 0;
+    __nv_bfloat16* Yb = nullptr;
+    float* Yf = nullptr;
+};
+
+template <int KZ, int KS, int CP, int COUTP, int CU>
+cudaError_t launch_conv_tc(stokes_net_s* n, Shape s, const ConvArgs& a) {
     using C = unet_tc::ConvCfg<KZ, KS, CP, COUTP>;
-    auto k = unet_tc::k_conv_tc<KZ, KS, CP, COUTP>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-    const unet_tc::TShape ts{s.B, s.D, s.H, s.W};
-    k<<<C::G::tiles(ts), 256, C::SMEM, n->s>>>(X, ts, Wp, bias, cout, relu, Yb, Yf);
+    auto k = unet_tc::k_conv_tc<KZ, KS, CP, COUTP, CU>;
+    static std::atomic<int> resident[MAX_DEVICES];
+    const unet_tc::TShape ts = C::G::shape(s.B, s.D, s.H, s.W);
+    const int G = persistent_ctas(n, k, C::SMEM, C::G::tiles(ts), 1 << 30, resident[n->device]);
+    k<<<G, 256, C::SMEM, n->s>>>(a.X, a.Xc, ts, a.Wp, a.bias, a.cout, a.relu, a.mask, a.Yb, a.Yf);
     return cudaGetLastError();
 }
 
-// one convolution on the tensor cores: input X with cp channels, packed
-// weights Wp with coutp rows
-cudaError_t conv_tc(stokes_net_s* n, int ks, int cp, int coutp, const __nv_bfloat16* X, Shape s,
-                    const __nv_bfloat16* Wp, const float* bias, int cout, int relu, __nv_bfloat16* Yb, float* Yf) {
-#define CONV_CASE(KZ_, KS_, CP_, CO_)                                                                      \
-    if (n->KZ == KZ_ && ks == KS_ && cp == CP_ && coutp == CO_)                                            \
-        return launch_conv_tc<KZ_, KS_, CP_, CO_>(n, X, s, Wp, bias, cout, relu, Yb, Yf);
+// one convolution on the tensor cores: cp input channels (cu of them from the
+// coarse tensor), packed weights with coutp rows
+cudaError_t conv_tc(stokes_net_s* n, int ks, int cp, int coutp, int cu, Shape s, const ConvArgs& a) {
+#define CONV_CASE(KZ_, KS_, CP_, CO_, CU_)                                     \
+    if (n->KZ == KZ_ && ks == KS_ && cp == CP_ && coutp == CO_ && cu == CU_)   \
+        return launch_conv_tc<KZ_, KS_, CP_, CO_, CU_>(n, s, a);
 #define CONV_CASES(KZ_)                                                                                    \
-    CONV_CASE(KZ_, 3, 8, 8) CONV_CASE(KZ_, 3, 16, 8) CONV_CASE(KZ_, 3, 8, 16) CONV_CASE(KZ_, 3, 16, 16)   \
-    CONV_CASE(KZ_, 3, 16, 32) CONV_CASE(KZ_, 3, 32, 32) CONV_CASE(KZ_, 3, 48, 16) CONV_CASE(KZ_, 3, 24, 8) \
-    CONV_CASE(KZ_, 3, 8, 24) CONV_CASE(KZ_, 3, 16, 48) CONV_CASE(KZ_, 3, 32, 16)                           \
-    CONV_CASE(KZ_, 1, 8, 8) CONV_CASE(KZ_, 1, 8, 16) CONV_CASE(KZ_, 1, 16, 8)
+    CONV_CASE(KZ_, 3, 8, 8, 0) CONV_CASE(KZ_, 3, 16, 8, 0) CONV_CASE(KZ_, 3, 8, 16, 0)                     \
+    CONV_CASE(KZ_, 3, 16, 16, 0) CONV_CASE(KZ_, 3, 16, 32, 0) CONV_CASE(KZ_, 3, 32, 32, 0)                 \
+    CONV_CASE(KZ_, 3, 48, 16, 32) CONV_CASE(KZ_, 3, 24, 8, 16) CONV_CASE(KZ_, 3, 8, 24, 0)                 \
+    CONV_CASE(KZ_, 3, 16, 48, 0) CONV_CASE(KZ_, 3, 32, 16, 0)                                              \
+    CONV_CASE(KZ_, 1, 8, 8, 0) CONV_CASE(KZ_, 1, 8, 16, 0) CONV_CASE(KZ_, 1, 16, 8, 0)
     CONV_CASES(3)
     CONV_CASES(1)
 #undef CONV_CASES
@@ -252,33 +367,32 @@ cudaError_t conv_tc(stokes_net_s* n, int ks, int cp, int coutp, const __nv_bfloa
     return cudaErrorInvalidValue;
 }
 
-template <int KZ, int KS, int CP, int COUTP>
-cudaError_t launch_wgrad_tc(stokes_net_s* n, const __nv_bfloat16* X, Shape s, const __nv_bfloat16* g16, int cin,
-                            int cout, float* dW, float* db) {
+template <int KZ, int KS, int CP, int COUTP, int CU>
+cudaError_t launch_wgrad_tc(stokes_net_s* n, const __nv_bfloat16* X, const __nv_bfloat16* Xc, Shape s,
+                            const __nv_bfloat16* g16, int cin, int cout, float* dW, float* db) {
     using C = unet_tc::WgCfg<KZ, KS, CP, COUTP>;
     static_assert(C::E + COUTP <= PART_STRIDE, "partial buffer too small");
-    auto k = unet_tc::k_wgrad_tc<KZ, KS, CP, COUTP>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-    int per = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 256, (int)C::SMEM);
-    const unet_tc::TShape ts{s.B, s.D, s.H, s.W};
-    const int G = std::min({C::G::tiles(ts), n->sms * std::max(per, 1), n->part_ctas});
-    k<<<G, 256, C::SMEM, n->s>>>(X, ts, g16, n->part);
+    static_assert(256 % COUTP == 0, "the bias sums deal whole channels to the threads");
+    auto k = unet_tc::k_wgrad_tc<KZ, KS, CP, COUTP, CU>;
+    static std::atomic<int> resident[MAX_DEVICES];
+    const unet_tc::TShape ts = C::G::shape(s.B, s.D, s.H, s.W);
+    const int G = persistent_ctas(n, k, C::SMEM, C::G::tiles(ts), n->part_ctas, resident[n->device]);
+    k<<<G, 256, C::SMEM, n->s>>>(X, Xc, ts, g16, n->part);
     const int tot = C::E + COUTP;
-    unet_tc::k_wgrad_reduce<<<(tot + 255) / 256, 256, 0, n->s>>>(n->part, G, C::G::TAPS, CP, COUTP, cin, cout, dW,
-                                                                  db);
+    unet_tc::k_wgrad_reduce<<<(tot + 31) / 32, 256, 0, n->s>>>(n->part, G, C::G::TAPS, CP, COUTP, cin, cout, dW, db);
     return cudaGetLastError();
 }
 
-cudaError_t wgrad_tc(stokes_net_s* n, int ks, int cp, int coutp, const __nv_bfloat16* X, Shape s,
-                     const __nv_bfloat16* g16, int cin, int cout, float* dW, float* db) {
-#define WG_CASE(KZ_, KS_, CP_, CO_)                                                                        \
-    if (n->KZ == KZ_ && ks == KS_ && cp == CP_ && coutp == CO_)                                            \
-        return launch_wgrad_tc<KZ_, KS_, CP_, CO_>(n, X, s, g16, cin, cout, dW, db);
+cudaError_t wgrad_tc(stokes_net_s* n, int ks, int cp, int coutp, int cu, const __nv_bfloat16* X,
+                     const __nv_bfloat16* Xc, Shape s, const __nv_bfloat16* g16, int cin, int cout, float* dW,
+                     float* db) {
+#define WG_CASE(KZ_, KS_, CP_, CO_, CU_)                                       \
+    if (n->KZ == KZ_ && ks == KS_ && cp == CP_ && coutp == CO_ && cu == CU_)   \
+        return launch_wgrad_tc<KZ_, KS_, CP_, CO_, CU_>(n, X, Xc, s, g16, cin, cout, dW, db);
 #define WG_CASES(KZ_)                                                                                      \
-    WG_CASE(KZ_, 3, 8, 8) WG_CASE(KZ_, 3, 16, 8) WG_CASE(KZ_, 3, 8, 16) WG_CASE(KZ_, 3, 16, 16)           \
-    WG_CASE(KZ_, 3, 16, 32) WG_CASE(KZ_, 3, 32, 32) WG_CASE(KZ_, 3, 48, 16) WG_CASE(KZ_, 3, 24, 8)         \
-    WG_CASE(KZ_, 1, 8, 8) WG_CASE(KZ_, 1, 8, 16)
+    WG_CASE(KZ_, 3, 8, 8, 0) WG_CASE(KZ_, 3, 16, 8, 0) WG_CASE(KZ_, 3, 8, 16, 0) WG_CASE(KZ_, 3, 16, 16, 0) \
+    WG_CASE(KZ_, 3, 16, 32, 0) WG_CASE(KZ_, 3, 32, 32, 0) WG_CASE(KZ_, 3, 48, 16, 32)                      \
+    WG_CASE(KZ_, 3, 24, 8, 16) WG_CASE(KZ_, 1, 8, 8, 0) WG_CASE(KZ_, 1, 8, 16, 0)
     WG_CASES(3)
     WG_CASES(1)
 #undef WG_CASES
@@ -288,103 +402,100 @@ cudaError_t wgrad_tc(stokes_net_s* n, int ks, int cp, int coutp, const __nv_bflo
 
 // pack the forward (and, for training, data-gradient) weights of every layer
 cudaError_t pack_weights(stokes_net_s* n, bool grad) {
+    unet_tc::PackList list{};
+    int m = 0, most = 0;
     for (size_t li = 0; li < n->L.size(); ++li) {
         const Conv& c = n->L[li];
-        const int taps = taps_of(n, c);
-        if (!n->wf_valid) {
-            const int rows = cp8(c.cout), tot = rows * taps * cp8(c.cin);
-            unet_tc::k_pack_weights<<<nblk(tot), 256, 0, n->s>>>(n->theta + c.w_off, taps, c.cin, c.cout, rows,
-                                                                  cp8(c.cin), 0, n->wf[li]);
-        }
-        if (grad) {
-            const int rows = cp8(c.cin), tot = rows * taps * cp8(c.cout);
-            unet_tc::k_pack_weights<<<nblk(tot), 256, 0, n->s>>>(n->theta + c.w_off, taps, c.cin, c.cout, rows,
-                                                                  cp8(c.cout), 1, n->wg[li]);
-        }
+        const int taps = taps_of(n, c), ci = cp8(c.cin), co = cp8(c.cout);
+        if (!n->wf_valid) list.l[m++] = {n->theta + c.w_off, n->wf[li], taps, c.cin, c.cout, co, ci, 0};
+        if (grad) list.l[m++] = {n->theta + c.w_off, n->wg[li], taps, c.cin, c.cout, ci, co, 1};
+        most = std::max(most, taps * ci * co);
     }
+    if (m) unet_tc::k_pack_weights<<<dim3(std::min(nblk(most), 32u), m), 256, 0, n->s>>>(list);
     n->wf_valid = true;
     return cudaGetLastError();
 }
 
-cudaError_t conv(stokes_net_s* n, int li, const __nv_bfloat16* X, Shape s, int relu, __nv_bfloat16* Yb, float* Yf) {
+// the decoder's first convolutions read their upsampled channels from the
+// coarse tensor
+int up_channels(int li) { return li == 6 ? 32 : li == 8 ? 16 : 0; }
+
+cudaError_t conv(stokes_net_s* n, int li, const __nv_bfloat16* X, Shape s, int relu, __nv_bfloat16* Yb, float* Yf,
+                 const __nv_bfloat16* Xc = nullptr) {
     const Conv& c = n->L[li];
-    return conv_tc(n, c.ks, cp8(c.cin), cp8(c.cout), X, s, n->wf[li], n->theta + c.b_off, c.cout, relu, Yb, Yf);
+    ConvArgs a;
+    a.X = X; a.Xc = Xc; a.Wp = n->wf[li]; a.bias = n->theta + c.b_off;
+    a.cout = c.cout; a.relu = relu; a.Yb = Yb; a.Yf = Yf;
+    return conv_tc(n, c.ks, cp8(c.cin), cp8(c.cout), up_channels(li), s, a);
 }
 
-// gradient step of layer li: dY (FP32, cout channels; the ReLU mask already
-// applied) -> BF16; weight and bias gradient from the layer input X; data
-// gradient into dX (FP32, cin channels) unless dX is null
-cudaError_t conv_backward(stokes_net_s* n, int li, const __nv_bfloat16* X, Shape s, const float* dY, float* dX) {
+// gradient step of layer li from its output gradient dY (BF16, cp(cout)
+// channels, the ReLU mask applied): weight and bias gradient from the layer
+// input X (and Xc); data gradient either through the ReLU of the layer input
+// as BF16 (dXb) or as FP32 (dXf), or neither
+cudaError_t conv_backward(stokes_net_s* n, int li, const __nv_bfloat16* X, Shape s, const __nv_bfloat16* dY,
+                          __nv_bfloat16* dXb, float* dXf, const __nv_bfloat16* Xc = nullptr) {
     const Conv& c = n->L[li];
-    unet_tc::k_to_bf16_pad<<<nblk(vox(s) * cp8(c.cout)), 256, 0, n->s>>>(dY, vox(s), c.cout, cp8(c.cout), n->g16);
-    cudaError_t e = wgrad_tc(n, c.ks, cp8(c.cin), cp8(c.cout), X, s, n->g16, c.cin, c.cout, n->grad + c.w_off,
-                             n->grad + c.b_off);
-    if (e != cudaSuccess || !dX) return e;
-    return conv_tc(n, c.ks, cp8(c.cout), cp8(c.cin), n->g16, s, n->wg[li], nullptr, c.cin, 0, nullptr, dX);
+    cudaError_t e = wgrad_tc(n, c.ks, cp8(c.cin), cp8(c.cout), up_channels(li), X, Xc, s, dY, c.cin, c.cout,
+                             n->grad + c.w_off, n->grad + c.b_off);
+    if (e != cudaSuccess || (!dXb && !dXf)) return e;
+    ConvArgs a;
+    a.X = dY; a.Wp = n->wg[li]; a.cout = c.cin;
+    a.mask = dXb ? X : nullptr; a.Yb = dXb; a.Yf = dXf;
+    return conv_tc(n, c.ks, cp8(c.cout), cp8(c.cin), 0, s, a);
 }
 
 Shape half(const Shape& s, int pz) { return Shape{s.B, pz ? s.D / 2 : s.D, s.H / 2, s.W / 2}; }
 
-cudaError_t forward(stokes_net_s* n, Shape s) {
+void to_bf16(stokes_net_s* n, const float* x, Shape s) {
+    const int cp = cp8(n->cin), per = 256 / (cp / 4);
+    unet_tc::k_to_bf16_pad<<<(unsigned)((vox(s) + per - 1) / per), 256, 0, n->s>>>(
+        x, vox(s), n->cin, cp, ((uintptr_t)x & 15u) == 0, n->xin);
+}
+
+// forward pass from xin; the output goes to `out` (FP32, cout channels)
+cudaError_t forward(stokes_net_s* n, Shape s, float* out) {
     const int pz = n->KZ == 3;
     if (!n->wf_valid && pack_weights(n, false) != cudaSuccess) return cudaGetLastError();
     Shape s1 = half(s, pz), s2 = half(s1, pz);
     cudaError_t e;
     if ((e = conv(n, 0, n->xin, s, 1, n->e0a, nullptr))) return e;
     if ((e = conv(n, 1, n->e0a, s, 1, n->e0, nullptr))) return e;
-    k_pool<<<nblk(vox(s1) * 8), 256, 0, n->s>>>(n->e0, s, 8, pz, n->p0);
+    k_pool<<<nblk(vox(s1)), 256, 0, n->s>>>(n->e0, s, s1, 8, pz, n->p0);
     if ((e = conv(n, 2, n->p0, s1, 1, n->e1a, nullptr))) return e;
     if ((e = conv(n, 3, n->e1a, s1, 1, n->e1, nullptr))) return e;
-    k_pool<<<nblk(vox(s2) * 16), 256, 0, n->s>>>(n->e1, s1, 16, pz, n->p1);
+    k_pool<<<nblk(vox(s2) * 2), 256, 0, n->s>>>(n->e1, s1, s2, 16, pz, n->p1);
     if ((e = conv(n, 4, n->p1, s2, 1, n->e2a, nullptr))) return e;
     if ((e = conv(n, 5, n->e2a, s2, 1, n->e2, nullptr))) return e;
-    k_up_concat<<<nblk(vox(s1) * 48), 256, 0, n->s>>>(n->e2, n->e1, s1, 32, 16, pz, n->c1);
-    if ((e = conv(n, 6, n->c1, s1, 1, n->d1a, nullptr))) return e;
+    if ((e = conv(n, 6, n->e1, s1, 1, n->d1a, nullptr, n->e2))) return e;
     if ((e = conv(n, 7, n->d1a, s1, 1, n->d1, nullptr))) return e;
-    k_up_concat<<<nblk(vox(s) * 24), 256, 0, n->s>>>(n->d1, n->e0, s, 16, 8, pz, n->c0);
-    if ((e = conv(n, 8, n->c0, s, 1, n->d0a, nullptr))) return e;
+    if ((e = conv(n, 8, n->e0, s, 1, n->d0a, nullptr, n->d1))) return e;
     if ((e = conv(n, 9, n->d0a, s, 1, n->d0, nullptr))) return e;
-    return conv(n, 10, n->d0, s, 0, nullptr, n->out);
+    return conv(n, 10, n->d0, s, 0, nullptr, out);
 }
 
-// backward from dL/dout (in g_a), accumulating parameter gradients in grad
+// backward from dL/dout (BF16 in gA), parameter gradients in grad
 cudaError_t backward(stokes_net_s* n, Shape s) {
     const int pz = n->KZ == 3;
     if (pack_weights(n, true) != cudaSuccess) return cudaGetLastError();
     Shape s1 = half(s, pz), s2 = half(s1, pz);
     cudaError_t e;
-    float *ga = n->g_a, *gb = n->g_b;
-    auto relu_b = [&](float* g, const __nv_bfloat16* y, int64_t nel) { k_relu_bwd<<<nblk(nel), 256, 0, n->s>>>(g, y, nel); };
-    // out (1x1, no ReLU): input d0
-    if ((e = conv_backward(n, 10, n->d0, s, ga, gb))) return e;                  // gb = d d0
-    relu_b(gb, n->d0, vox(s) * 8);
-    if ((e = conv_backward(n, 9, n->d0a, s, gb, ga))) return e;                   // ga = d d0a
-    relu_b(ga, n->d0a, vox(s) * 8);
-    if ((e = conv_backward(n, 8, n->c0, s, ga, gb))) return e;                   // gb = d c0 (24 ch)
-    cudaMemsetAsync(n->g_skip0, 0, sizeof(float) * vox(s) * 8, n->s);
-    k_up_concat_adj<<<nblk(std::max(vox(s1) * 16, vox(s) * 8)), 256, 0, n->s>>>(gb, s, 16, 8, pz, ga, n->g_skip0);
-    // ga = d d1 (16 ch at s1)
-    relu_b(ga, n->d1, vox(s1) * 16);
-    if ((e = conv_backward(n, 7, n->d1a, s1, ga, gb))) return e;                  // gb = d d1a
-    relu_b(gb, n->d1a, vox(s1) * 16);
-    if ((e = conv_backward(n, 6, n->c1, s1, gb, ga))) return e;                  // ga = d c1 (48 ch at s1)
-    cudaMemsetAsync(n->g_skip1, 0, sizeof(float) * vox(s1) * 16, n->s);
-    k_up_concat_adj<<<nblk(std::max(vox(s2) * 32, vox(s1) * 16)), 256, 0, n->s>>>(ga, s1, 32, 16, pz, gb, n->g_skip1);
-    // gb = d e2 (32 ch at s2)
-    relu_b(gb, n->e2, vox(s2) * 32);
-    if ((e = conv_backward(n, 5, n->e2a, s2, gb, ga))) return e;                  // ga = d e2a
-    relu_b(ga, n->e2a, vox(s2) * 32);
-    if ((e = conv_backward(n, 4, n->p1, s2, ga, gb))) return e;                  // gb = d p1 (16 ch at s2)
-    k_pool_adj<<<nblk(vox(s1) * 16), 256, 0, n->s>>>(gb, s1, 16, pz, n->g_skip1);   // += into d e1
-    relu_b(n->g_skip1, n->e1, vox(s1) * 16);
-    if ((e = conv_backward(n, 3, n->e1a, s1, n->g_skip1, ga))) return e;          // ga = d e1a
-    relu_b(ga, n->e1a, vox(s1) * 16);
-    if ((e = conv_backward(n, 2, n->p0, s1, ga, gb))) return e;                  // gb = d p0 (8 ch at s1)
-    k_pool_adj<<<nblk(vox(s) * 8), 256, 0, n->s>>>(gb, s, 8, pz, n->g_skip0);      // += into d e0
-    relu_b(n->g_skip0, n->e0, vox(s) * 8);
-    if ((e = conv_backward(n, 1, n->e0a, s, n->g_skip0, ga))) return e;           // ga = d e0a
-    relu_b(ga, n->e0a, vox(s) * 8);
-    return conv_backward(n, 0, n->xin, s, ga, nullptr);
+    __nv_bfloat16 *gA = n->gA, *gB = n->gB;
+    if ((e = conv_backward(n, 10, n->d0, s, gA, gB, nullptr))) return e;              // gB = d d0
+    if ((e = conv_backward(n, 9, n->d0a, s, gB, gA, nullptr))) return e;              // gA = d d0a
+    if ((e = conv_backward(n, 8, n->e0, s, gA, nullptr, n->g_c0, n->d1))) return e;   // g_c0 = d [up d1, e0]
+    k_up_adj<<<nblk(vox(s1) * 2), 256, 0, n->s>>>(n->g_c0, s, s1, 16, 24, pz, n->d1, gB);         // gB = d d1
+    if ((e = conv_backward(n, 7, n->d1a, s1, gB, gA, nullptr))) return e;             // gA = d d1a
+    if ((e = conv_backward(n, 6, n->e1, s1, gA, nullptr, n->g_c1, n->e2))) return e;  // g_c1 = d [up e2, e1]
+    k_up_adj<<<nblk(vox(s2) * 4), 256, 0, n->s>>>(n->g_c1, s1, s2, 32, 48, pz, n->e2, gB);        // gB = d e2
+    if ((e = conv_backward(n, 5, n->e2a, s2, gB, gA, nullptr))) return e;             // gA = d e2a
+    if ((e = conv_backward(n, 4, n->p1, s2, gA, nullptr, n->g_p1))) return e;         // g_p1 = d p1
+    k_skip_pool_adj<<<nblk(vox(s1) * 2), 256, 0, n->s>>>(n->g_c1, n->g_p1, s1, s2, 16, 32, 48, pz, n->e1, gB);  // d e1
+    if ((e = conv_backward(n, 3, n->e1a, s1, gB, gA, nullptr))) return e;             // gA = d e1a
+    if ((e = conv_backward(n, 2, n->p0, s1, gA, nullptr, n->g_p0))) return e;         // g_p0 = d p0
+    k_skip_pool_adj<<<nblk(vox(s)), 256, 0, n->s>>>(n->g_c0, n->g_p0, s, s1, 8, 16, 24, pz, n->e0, gB);         // d e0
+    if ((e = conv_backward(n, 1, n->e0a, s, gB, gA, nullptr))) return e;              // gA = d e0a
+    return conv_backward(n, 0, n->xin, s, gA, nullptr, nullptr);
 }
 
 }  // namespace
@@ -436,21 +547,23 @@ stokes_status stokes_net_create(stokes_net* out, int dim, int cin, int cout, int
     }
     int dev = 0;
     cudaGetDevice(&dev);
+    n->device = dev >= 0 && dev < MAX_DEVICES ? dev : 0;
     cudaDeviceGetAttribute(&n->sms, cudaDevAttrMultiProcessorCount, dev);
     n->part_ctas = 2 * std::max(n->sms, 1);
     A((void**)&n->part, 4 * (size_t)n->part_ctas * PART_STRIDE);
-    A((void**)&n->g16, 2 * V * 8);
+    // the levels hold at most V, V / 4 and V / 16 voxels (2D; fewer in 3D)
+    A((void**)&n->gA, 2 * V * 16);
+    A((void**)&n->gB, 2 * V * 16);
     A((void**)&n->xin, 2 * V * cp8(cin));
     __nv_bfloat16** full8[] = {&n->e0a, &n->e0, &n->d0a, &n->d0};
     for (auto p : full8) A((void**)p, 2 * V * 8);
-    A((void**)&n->c0, 2 * V * 24);
-    __nv_bfloat16** half16[] = {&n->p0, &n->e1a, &n->e1, &n->d1a, &n->d1};
-    for (auto p : half16) A((void**)p, 2 * V * 16);          // generous (V/4 or V/8 needed)
-    A((void**)&n->c1, 2 * V * 48 / 2);
-    A((void**)&n->p1, 2 * V * 16); A((void**)&n->e2a, 2 * V * 32 / 4); A((void**)&n->e2, 2 * V * 32 / 4);
+    __nv_bfloat16** half16[] = {&n->p0, &n->e1a, &n->e1, &n->p1, &n->d1a, &n->d1};
+    for (auto p : half16) A((void**)p, 2 * (V / 4 + 1) * 16);
+    A((void**)&n->e2a, 2 * (V / 16 + 1) * 32); A((void**)&n->e2, 2 * (V / 16 + 1) * 32);
     A((void**)&n->out, 4 * V * cout);
-    A((void**)&n->g_a, 4 * V * 48); A((void**)&n->g_b, 4 * V * 48); A((void**)&n->g_c, 4 * V * 48);
-    A((void**)&n->g_skip0, 4 * V * 8); A((void**)&n->g_skip1, 4 * V * 16);
+    A((void**)&n->g_c0, 4 * V * 24); A((void**)&n->g_c1, 4 * (V / 4 + 1) * 48);
+    A((void**)&n->g_p0, 4 * (V / 4 + 1) * 8); A((void**)&n->g_p1, 4 * (V / 16 + 1) * 16);
+    A((void**)&n->fac, 16 * 1024);
     A((void**)&n->sums, 16 * 1024 + 16 * 1024 * LOSS_BLOCKS);   // sums, then the per-block partials
     if (e != cudaSuccess) { stokes_net_destroy(n); return STOKES_ERR_CUDA; }
     *out = n;
@@ -484,10 +597,8 @@ static bool shape_ok(stokes_net n, int B, int D, int H, int W) {
 stokes_status stokes_net_forward(stokes_net n, int B, int D, int H, int W, const float* x, float* y) {
     if (!n || !x || !y || !shape_ok(n, B, D, H, W)) return STOKES_ERR_ARG;
     Shape s{B, D, H, W};
-    unet_tc::k_to_bf16_pad<<<nblk(vox(s) * cp8(n->cin)), 256, 0, n->s>>>(x, vox(s), n->cin, cp8(n->cin), n->xin);
-    if (forward(n, s) != cudaSuccess) return STOKES_ERR_CUDA;
-    if (cudaMemcpyAsync(y, n->out, 4 * vox(s) * n->cout, cudaMemcpyDeviceToDevice, n->s) != cudaSuccess)
-        return STOKES_ERR_CUDA;
+    to_bf16(n, x, s);
+    if (forward(n, s, y) != cudaSuccess) return STOKES_ERR_CUDA;
     return cudaStreamSynchronize(n->s) == cudaSuccess ? STOKES_OK : STOKES_ERR_CUDA;
 }
 
@@ -497,12 +608,16 @@ stokes_status stokes_net_gradient(stokes_net n, int B, int D, int H, int W, cons
                                   double* loss, float* grad_host) {
     if (!n || !x || !y || !shape_ok(n, B, D, H, W) || B > 1024) return STOKES_ERR_ARG;
     Shape s{B, D, H, W};
-    unet_tc::k_to_bf16_pad<<<nblk(vox(s) * cp8(n->cin)), 256, 0, n->s>>>(x, vox(s), n->cin, cp8(n->cin), n->xin);
-    if (forward(n, s) != cudaSuccess) return STOKES_ERR_CUDA;
-    int64_t per = (int64_t)D * H * W * n->cout;
-    k_loss_partials<<<dim3(LOSS_BLOCKS, B), 256, 0, n->s>>>(n->out, y, per, n->sums + 2 * 1024);
-    k_loss_finish<<<(B + 127) / 128, 128, 0, n->s>>>(n->sums + 2 * 1024, B, n->sums);
-    k_loss_grad<<<nblk(per * B), 256, 0, n->s>>>(n->out, y, per, B, n->sums, n->g_a);
+    to_bf16(n, x, s);
+    if (forward(n, s, n->out) != cudaSuccess) return STOKES_ERR_CUDA;
+    const int64_t nv = (int64_t)D * H * W, per = nv * n->cout;
+    const int cp = cp8(n->cout);
+    // eight elements per thread or more
+    const int lb = (int)std::min<int64_t>(LOSS_BLOCKS, (per + 2047) / 2048);
+    k_loss_partials<<<dim3(lb, B), 256, 0, n->s>>>(n->out, y, per, n->sums + 2 * 1024);
+    k_loss_finish<<<B, 32, 0, n->s>>>(n->sums + 2 * 1024, lb, B, n->sums, n->fac);
+    const int vpb = 256 / (cp / 4);
+    k_loss_grad<<<dim3((unsigned)((nv + vpb - 1) / vpb), B), 256, 0, n->s>>>(n->out, y, nv, n->cout, cp, n->fac, n->gA);
     cudaMemsetAsync(n->grad, 0, 4 * n->np, n->s);
     if (backward(n, s) != cudaSuccess) return STOKES_ERR_CUDA;
     std::vector<double> sums(2 * B);

@@ -443,7 +443,7 @@ class Net:
 
     def forward(self, x, shape):
         B, D, H, W = shape
-        y = torch.zeros(B * D * H * W * self.cout, dtype=torch.float32, device="cuda")
+        y = torch.empty(B * D * H * W * self.cout, dtype=torch.float32, device="cuda")   # written in full
         st = self.lib.stokes_net_forward(self.h, B, D, H, W, _dev(x, torch.float32).data_ptr(), y.data_ptr())
         if st != 0:
             raise StokesError(st, "stokes_net_forward failed")

@@ -179,7 +179,7 @@ stokes_status stokes_create(stokes_ctx* out, const stokes_grid* g, void* stream)
     size_t wb = 0;
     auto add = [&](size_t bytes) { size_t o = wb; wb += round_up((int64_t)bytes, 256); return o; };
     size_t oWL = add(sizeof(double) * S * c.nk), oWF = add(sizeof(double) * S * c.nk);
-    size_t oFF = add(S * c.nd), oEW = add(sizeof(double) * S * c.nd), oK = add(sizeof(double) * S * c.nd);
+    size_t oFF = add(S * c.nd), oEW = add(sizeof(double) * S * c.nd);
     size_t oRec = add(sizeof(double) * S * c.nd), oUbc = add(sizeof(double) * S * c.nd);
     size_t oAct = add(S * c.nsite);
     size_t oC64 = add(sizeof(double) * S * c.ncoef), oC32 = add(sizeof(float) * S * c.ncoef);
@@ -203,7 +203,7 @@ stokes_status stokes_create(stokes_ctx* out, const stokes_grid* g, void* stream)
         for (int d = 0; d < c.nd; ++d) {
             A.fflag[d] = (uint8_t*)(base + oFF) + d * S;
             A.effWF[d] = (double*)(base + oEW) + d * S;
-            A.K64[d] = (double*)(base + oK) + d * S;
+            A.K64[d] = (double*)(base + oC64) + (c.ncoef - c.nd + d) * S;    // the last coefficient fields
             A.rec[d] = (double*)(base + oRec) + d * S;
             A.ubc[d] = (double*)(base + oUbc) + d * S;
         }
@@ -221,6 +221,7 @@ stokes_status stokes_create(stokes_ctx* out, const stokes_grid* g, void* stream)
     }
     const int64_t V = (int64_t)c.nf * S;
     if (e == cudaSuccess) e = dalloc(c, (void**)&c.tiles, sizeof(int) * c.ntiles_all);
+    if (e == cudaSuccess) e = dalloc(c, (void**)&c.sign_bits, sign_bits_bytes(L));
     if (e == cudaSuccess) e = dalloc(c, (void**)&c.d_ntiles, sizeof(int));
     if (e == cudaSuccess) e = dalloc(c, (void**)&c.units, sizeof(int) * std::max(c.nunits_all, 1));
     if (e == cudaSuccess) e = dalloc(c, (void**)&c.d_nunits, sizeof(int));

@@ -75,6 +75,7 @@ struct Ctx {
     DevArrays A{};
     void* weight_block = nullptr;
     size_t weight_bytes = 0;
+    uint32_t* sign_bits = nullptr;  // 3D: scratch of the weight build (k_sign_bits)
     // solver state
     CgScalars* sc = nullptr;     // [0] inner/plain CG, [1] outer
     CgScalars* h_sc = nullptr;   // pinned host mirror
@@ -110,7 +111,10 @@ struct Ctx {
         a.zt = unit_zt;
         return a;
     }
-    cudaError_t zero_weights() { return cudaMemsetAsync(weight_block, 0, weight_bytes, stream); }
+    // the tile flags and unit masks are the last part of the weight block
+    cudaError_t zero_tile_flags() {
+        return cudaMemsetAsync(A.tile_flag, 0, weight_bytes - (size_t)(A.tile_flag - (uint8_t*)weight_block), stream);
+    }
     template <class C> Coef<C> coef() const;
     int64_t vec_elems() const { return (int64_t)nf * L.stride; }
 };

@@ -89,6 +89,7 @@ void set_error(Ctx* c, const std::string& m);
 // weights.cu
 cudaError_t launch_build_weights(Ctx* c, const double* phiL, const double* phiS, const double* const* rho,
                                  const double* const* mu, const double* const* ubc);
+size_t sign_bits_bytes(const Layout& L);
 // rhs_recover.cu
 cudaError_t launch_rhs(Ctx* c, const double* const* ustar, double* b);
 cudaError_t launch_recover(Ctx* c, const double* const* ustar, const double* x, double* const* uout);

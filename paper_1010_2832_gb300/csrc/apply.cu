@@ -25,40 +25,6 @@
 
 namespace stk {
 
-// Block reduction of one double per thread into partial[blockIdx.x], then the
-// last block sums all partials (index order) and calls fin(total).
-template <int NT, class Fin>
-__device__ void block_partial_and_finish(double v, double* partial, unsigned* counter, int nblocks, Fin fin) {
-    __shared__ double red[NT / 32];
-    __shared__ bool last;
-    v = warp_sum(v);
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) red[w] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int q = 0; q < NT / 32; ++q) s += red[q];
-        partial[blockIdx.x] = s;
-        __threadfence();
-        unsigned prev = atomicAdd(counter, 1u);
-        last = (prev == (unsigned)nblocks - 1u);
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    double s = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += NT) s += ((volatile double*)partial)[b];
-    s = warp_sum(s);
-    if (lane == 0) red[w] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int q = 0; q < NT / 32; ++q) tot += red[q];
-        fin(tot);
-        *counter = 0u;
-    }
-}
-
 // ------------------------------- 2D -----------------------------------------
 // Everything one thread loads for one 2D tile (32 x 8 slots, 256 threads):
 // two staging positions of the (8+2) x (32+2) halo region, two face
@@ -204,10 +170,10 @@ __global__ void __launch_bounds__(256, MINB) k_apply2d(Layout L, const int* __re
         __syncthreads();                         // the next tile's staging reuses shared memory
     }
     if (MODE != MODE_PLAIN) {
-        double v = acc.warp();
-        if ((t & 31) != 0) v = 0.0;
         CgScalars* sc = args.sc;
-        block_partial_and_finish<256>(v, args.partial, args.counter, gridDim.x, [&](double tot) {
+        const Acc<T> sums[1] = {acc};
+        block_sums<T, 1>(sums, args.partial, args.counter, gridDim.x, [&](const double (&tots)[1]) {
+            const double tot = tots[0];
             if (MODE == MODE_RESID) { sc->rr = tot; return; }
             sc->pq = tot;
             if (!(tot > 0.0) || !isfinite(tot)) { sc->done = 1; sc->status = (isfinite(tot) ? STOKES_ERR_BREAKDOWN : STOKES_ERR_NONFINITE); }
@@ -549,10 +515,10 @@ __global__ void __launch_bounds__(256, 2) k_apply2d_v4(Layout L, const int* __re
         gsync();                                 // the next tile's staging reuses the group's shared memory
     }
     if (MODE != MODE_PLAIN) {
-        double v = acc.warp();
-        if ((threadIdx.x & 31) != 0) v = 0.0;
         CgScalars* sc = args.sc;
-        block_partial_and_finish<256>(v, args.partial, args.counter, gridDim.x, [&](double tot) {
+        const Acc<float> sums[1] = {acc};
+        block_sums<float, 1>(sums, args.partial, args.counter, gridDim.x, [&](const double (&tots)[1]) {
+            const double tot = tots[0];
             if (MODE == MODE_RESID) { sc->rr = tot; return; }
             sc->pq = tot;
             if (!(tot > 0.0) || !isfinite(tot)) { sc->done = 1; sc->status = (isfinite(tot) ? STOKES_ERR_BREAKDOWN : STOKES_ERR_NONFINITE); }
@@ -821,10 +787,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
         // orders them
     }
     if (MODE != MODE_PLAIN) {
-        double v = acc.warp();
-        if ((threadIdx.x & 31) != 0) v = 0.0;
         CgScalars* sc = args.sc;
-        block_partial_and_finish<256>(v, args.partial, args.counter, gridDim.x, [&](double tot) {
+        const Acc<T> sums[1] = {acc};
+        block_sums<T, 1>(sums, args.partial, args.counter, gridDim.x, [&](const double (&tots)[1]) {
+            const double tot = tots[0];
             if (MODE == MODE_RESID) { sc->rr = tot; return; }
             sc->pq = tot;
             if (!(tot > 0.0) || !isfinite(tot)) { sc->done = 1; sc->status = (isfinite(tot) ? STOKES_ERR_BREAKDOWN : STOKES_ERR_NONFINITE); }

@@ -2,29 +2,9 @@
 // persistent batched solver).  See apply.cu for the method and the modes.
 #pragma once
 #include "internal.cuh"
+#include "reduce.cuh"
 
 namespace stk {
-
-template <class T> struct Acc;
-template <> struct Acc<double> {
-    double s = 0.0;
-    __device__ void add(double a, double b) { s = fma(a, b, s); }
-    __device__ double warp() { return warp_sum(s); }
-};
-// FP32 vectors: products and sums kept as float-float pairs (TwoProd via FMA,
-// TwoSum) so the partial is accurate to ~2^-44 relative without FP64 math.
-template <> struct Acc<float> {
-    float hi = 0.f, lo = 0.f;
-    __device__ void add(float a, float b) {
-        float p = a * b;
-        float e = fmaf(a, b, -p);
-        float s, t;
-        two_sum(hi, p, s, t);
-        lo += t + e;
-        hi = s;
-    }
-    __device__ double warp() { return warp_sum_ff(hi, lo); }
-};
 
 template <class T, class C> __device__ __forceinline__ T ld(const C* p, int64_t o);
 template <> __device__ __forceinline__ double ld<double, double>(const double* p, int64_t o) { return __ldg(p + o); }

@@ -23,6 +23,7 @@
 #include <vector>
 #include "internal.cuh"
 #include "ctx.cuh"
+#include "reduce.cuh"
 
 namespace stk {
 
@@ -43,63 +44,6 @@ __device__ __forceinline__ int64_t tile_row_off(const Layout& L, int tile, int r
     return L.off(tcx * TX, tr * TY3 + row % TY3, tq * TZ3 + row / TY3);
 }
 
-template <class T> struct AccT;
-template <> struct AccT<double> {
-    double s = 0.0;
-    __device__ void add(double a, double b) { s = fma(a, b, s); }
-    __device__ double warp() { return warp_sum(s); }
-};
-template <> struct AccT<float> {
-    float hi = 0.f, lo = 0.f;
-    __device__ void add(float a, float b) {
-        float p = a * b;
-        float e = fmaf(a, b, -p);
-        float s, t;
-        two_sum(hi, p, s, t);
-        lo += t + e;
-        hi = s;
-    }
-    __device__ double warp() { return warp_sum_ff(hi, lo); }
-};
-
-// Two partial sums per block; the last block to finish reduces both.
-template <class Fin>
-__device__ void block_partial2(double v0, double v1, double* partial, unsigned* counter, int nblocks, Fin fin) {
-    __shared__ double red[2][8];
-    __shared__ bool last;
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) { red[0][w] = v0; red[1][w] = v1; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s0 = 0.0, s1 = 0.0;
-        for (int q = 0; q < 8; ++q) { s0 += red[0][q]; s1 += red[1][q]; }
-        partial[2 * blockIdx.x] = s0;
-        partial[2 * blockIdx.x + 1] = s1;
-        __threadfence();
-        unsigned prev = atomicAdd(counter, 1u);
-        last = (prev == (unsigned)nblocks - 1u);
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    double s0 = 0.0, s1 = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += 256) {
-        s0 += ((volatile double*)partial)[2 * b];
-        s1 += ((volatile double*)partial)[2 * b + 1];
-    }
-    s0 = warp_sum(s0);
-    s1 = warp_sum(s1);
-    __syncthreads();
-    if (lane == 0) { red[0][w] = s0; red[1][w] = s1; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t0 = 0.0, t1 = 0.0;
-        for (int q = 0; q < 8; ++q) { t0 += red[0][q]; t1 += red[1][q]; }
-        fin(t0, t1);
-        *counter = 0u;
-    }
-}
-
 // init: r = T(scale * r64), z = minv r, x = 0, p0 = 0; rho = r.z, rr0 = r.r
 template <class T>
 __global__ void __launch_bounds__(256) k_cg_init(Layout L, const int* __restrict__ tiles, int nf, const double* r64,
@@ -109,7 +53,8 @@ __global__ void __launch_bounds__(256) k_cg_init(Layout L, const int* __restrict
     const int tile = tiles[blockIdx.x];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const T scale = (T)sc->scale;
-    AccT<T> rz, rr;
+    Acc<T> dots[2];
+    Acc<T>&rz = dots[0], &rr = dots[1];
     const int nrow = tile_rows(L);
     for (int row = warp; row < nrow; row += 8) {
         int64_t o = tile_row_off(L, tile, row) + lane;
@@ -121,8 +66,8 @@ __global__ void __launch_bounds__(256) k_cg_init(Layout L, const int* __restrict
             rz.add(r, z); rr.add(r, r);
         }
     }
-    double a = rz.warp(), b = rr.warp();
-    block_partial2(a, b, partial, counter, nblocks, [&](double trz, double trr) {
+    block_sums<T, 2>(dots, partial, counter, nblocks, [&](const double (&tot)[2]) {
+        const double trz = tot[0], trr = tot[1];
         sc->rz = trz; sc->rr = trr; sc->rr0 = trr;
         sc->tol2 = sc->tol_rel * sc->tol_rel * trr;
         sc->beta = 0.0; sc->iter = 0; sc->status = 0;
@@ -144,7 +89,8 @@ __global__ void __launch_bounds__(256) k_cg_update(Layout L, const int* __restri
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const T alpha = (T)sc->alpha;
-    AccT<T> rz, rr;
+    Acc<T> dots[2];
+    Acc<T>&rz = dots[0], &rr = dots[1];
     const int nrow = tile_rows(L);
     T* __restrict__ X = w.x;
     T* __restrict__ Rr = w.r;
@@ -177,8 +123,8 @@ __global__ void __launch_bounds__(256) k_cg_update(Layout L, const int* __restri
         }
     }
     }
-    double a = rz.warp(), b = rr.warp();
-    block_partial2(a, b, partial, counter, gridDim.x, [&](double trz, double trr) {
+    block_sums<T, 2>(dots, partial, counter, gridDim.x, [&](const double (&tot)[2]) {
+        const double trz = tot[0], trr = tot[1];
         sc->rr = trr;
         sc->iter += 1;
         if (!isfinite(trr) || !isfinite(trz)) { sc->done = 1; sc->status = STOKES_ERR_NONFINITE; }
@@ -231,7 +177,8 @@ __global__ void __launch_bounds__(256, UPD ? 3 : 5) k_sw_finish(Layout L, const 
         if (use_cond && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
         return;
     }
-    AccT<float> rz, rr;
+    Acc<float> dots[2];
+    Acc<float>&rz = dots[0], &rr = dots[1];
     // persistent over the tile list, two tiles per round (tile k and tile
     // k + gridDim.x): the loads of both slots are issued before either is
     // summed; one block reduction per CTA
@@ -253,7 +200,8 @@ __global__ void __launch_bounds__(256, UPD ? 3 : 5) k_sw_finish(Layout L, const 
         sw_gather_finish(L, g0, w.z, rz, rr, UPD ? &u0 : nullptr, alpha, w.r, w.x);
         if (k2 < ntiles) sw_gather_finish(L, g1, w.z, rz, rr, UPD ? &u1 : nullptr, alpha, w.r, w.x);
     }
-    block_partial2(rz.warp(), rr.warp(), partial, counter, gridDim.x, [&](double trz, double trr) {
+    block_sums<float, 2>(dots, partial, counter, gridDim.x, [&](const double (&tot)[2]) {
+        const double trz = tot[0], trr = tot[1];
         if (INIT) {
             const bool timed_out = sc->status == STOKES_ERR_TIMEOUT;   // set by a local solve
             sc->rz = trz; sc->rr = trr; sc->rr0 = trr;
@@ -408,7 +356,8 @@ __global__ void __launch_bounds__(256) k_outer_init(Layout L, const int* __restr
                                                     unsigned* counter, int nblocks) {
     const int tile = tiles[blockIdx.x];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double s = 0.0;
+    Acc<double> dots[1];
+    double& s = dots[0].s;
     const int nrow = tile_rows(L);
     for (int row = warp; row < nrow; row += 8) {
         int64_t o = tile_row_off(L, tile, row) + lane;
@@ -419,8 +368,8 @@ __global__ void __launch_bounds__(256) k_outer_init(Layout L, const int* __restr
             s = fma(v, v, s);
         }
     }
-    double a = warp_sum(s);
-    block_partial2(a, 0.0, partial, counter, nblocks, [&](double t0, double) {
+    block_sums<double, 1>(dots, partial, counter, nblocks, [&](const double (&tot)[1]) {
+        const double t0 = tot[0];
         so->rr = t0; so->rr0 = t0; so->iter = 0; so->status = 0; so->done = 0;
     });
 }

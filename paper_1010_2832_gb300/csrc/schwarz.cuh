@@ -454,7 +454,7 @@ __device__ __forceinline__ void sw_gather_load(const Layout& L, const DevArrays&
 // With an update u (and alpha): r -= alpha q and x += alpha p are written
 // first, and z, r.z, r.r use the new r.
 __device__ __forceinline__ void sw_gather_finish(const Layout& L, SwGather& g, float* __restrict__ z,
-                                                 AccT<float>& rz, AccT<float>& r2, const SwUpdate* u = nullptr,
+                                                 Acc<float>& rz, Acc<float>& r2, const SwUpdate* u = nullptr,
                                                  float alpha = 0.f, float* __restrict__ r = nullptr,
                                                  float* __restrict__ x = nullptr) {
 #pragma unroll

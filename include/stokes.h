@@ -184,8 +184,9 @@ typedef struct {
                           4x4 slots plus a one-slot ring, exact local solves
                           (inverse factors stored in FP16 with a FP32 scale
                           per row, FP32 inner CG)                             */
-    int use_graph;     /* 1: CG loop in a device-side CUDA graph (conditional
-                          while node); 0: host-driven chunks of check_every
+    int use_graph;     /* 1: CG loop on the device, in one cooperative kernel
+                          for small 2D systems, else in a CUDA graph
+                          (conditional while node); 0: host-driven chunks of check_every
                           iterations launched one kernel at a time (for
                           profilers that cannot enter conditional graphs)   */
     int wait_test;     /* test hook for the bounded device-side waits, 0 in

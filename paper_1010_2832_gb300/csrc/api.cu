@@ -7,6 +7,7 @@
 #include <string>
 #include "internal.cuh"
 #include "ctx.cuh"
+#include "grid_gather.cuh"
 
 using namespace stk;
 
@@ -187,6 +188,7 @@ stokes_status stokes_create(stokes_ctx* out, const stokes_grid* g, void* stream)
     size_t oP16 = add(g->dim == 2 ? sizeof(uint32_t) * S * 3 : 4);
     size_t oQ16 = add(g->dim == 3 ? sizeof(uint2) * S * 2 : 8);
     size_t oM64 = add(sizeof(double) * S * c.nf), oM32 = add(sizeof(float) * S * c.nf);
+    size_t oGather = add(GATHER_BYTES), oSign = add(sign_bits_bytes(L));
     size_t oTF = add(c.ntiles_all);
     size_t oTF4 = add(g->dim == 2 ? (size_t)L.ntx * (L.R / 4) : 1);
     c.nunits_all = g->dim == 3 ? L.ntx * units_y(L.nty) * units_z(L.ntz, 1) : 0;
@@ -218,10 +220,11 @@ stokes_status stokes_create(stokes_ctx* out, const stokes_grid* g, void* stream)
         A.tile_flag = (uint8_t*)(base + oTF);
         A.tile_flag4 = (uint8_t*)(base + oTF4);
         A.unit_mask = (uint8_t*)(base + oUM);
+        c.gather = (unsigned long long*)(base + oGather);
+        c.sign_bits = (uint32_t*)(base + oSign);
     }
     const int64_t V = (int64_t)c.nf * S;
     if (e == cudaSuccess) e = dalloc(c, (void**)&c.tiles, sizeof(int) * c.ntiles_all);
-    if (e == cudaSuccess) e = dalloc(c, (void**)&c.sign_bits, sign_bits_bytes(L));
     if (e == cudaSuccess) e = dalloc(c, (void**)&c.d_ntiles, sizeof(int));
     if (e == cudaSuccess) e = dalloc(c, (void**)&c.units, sizeof(int) * std::max(c.nunits_all, 1));
     if (e == cudaSuccess) e = dalloc(c, (void**)&c.d_nunits, sizeof(int));

@@ -81,6 +81,8 @@ struct Ctx {
     CgScalars* h_sc = nullptr;   // pinned host mirror
     double* partial = nullptr;   // per-block partials (2 arrays)
     unsigned* counter = nullptr;
+    unsigned long long* gather = nullptr;   // slots of the cooperative CG kernels (grid_gather.cuh)
+    unsigned long long* zwords = nullptr;   // 2D: boundary values between their CTAs, allocated on first use
     CgWork<double> w64;
     CgWork<float> w32;
     double* b64 = nullptr;       // rhs (solve_step)
@@ -142,6 +144,11 @@ template <> inline Coef<__nv_bfloat16> Ctx::coef<__nv_bfloat16>() const {
 template <class T, class C>
 cudaError_t launch_apply_mode(const Layout& L, const int* tiles, int ntiles, const Coef<C>& cf, const T* x, T* y,
                               int mode, const ApplyArgs& a, cudaStream_t s);
+
+// cgloop.cu: the whole Jacobi-PCG loop in one cooperative kernel, for systems
+// small enough (*taken says whether it was launched)
+template <class T, class C>
+cudaError_t launch_cg_loop(Ctx* c, CgWork<T>& w, const T* minv, const Coef<C>& cf, int update_ctas, bool* taken);
 
 }  // namespace stk
 

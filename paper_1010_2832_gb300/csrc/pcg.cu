@@ -7,9 +7,10 @@
 //   iterate   [apply, CG mode]  p = z + beta p_old, q = A p, alpha = rho / p.q
 //             [update]          x += alpha p, r -= alpha q, z = M^-1 r,
 //                               rho' = r.z, beta = rho'/rho, stop on r.r <= tol2
-// The loop runs on the device as a CUDA graph with a conditional while node
-// whose condition the update kernel clears when the solve is done, so the
-// host is involved once per inner solve.
+// The loop runs on the device: small 2D systems in one cooperative kernel
+// (cgloop.cu), the others as a CUDA graph with a conditional while node whose
+// condition the update kernel clears when the solve is done, so the host is
+// involved once per inner solve.
 //
 // Outer loop (FP64): x64 += d / scale, r64 = b - A64 x64 recomputed from
 // scratch with the FP64 operator; stop when ||r64|| <= tol ||b||.  In FP64
@@ -443,6 +444,10 @@ static cudaError_t run_inner(Ctx* c, int prec_slot, CgWork<T>& w, const T* minv,
                              int chunk) {
     cudaError_t e;
     if (use_graph) {
+        // small systems: the whole loop in one cooperative kernel
+        bool taken = false;
+        e = launch_cg_loop<T, C>(c, w, minv, cf, persist_grid((const void*)k_cg_update<T>, 1 << 30), &taken);
+        if (taken || e != cudaSuccess) return e;
         cudaGraphExec_t& ge = c->graph[prec_slot];
         if (!ge) {
             if ((e = build_inner_graph<T, C>(c, w, minv, cf, c->sc, &ge)) != cudaSuccess) return e;

@@ -70,6 +70,24 @@ __device__ __forceinline__ void tile2_load(const Layout& L, int c0, int r0, cons
     d.odn = ld<T, C>(cf.f[3], o);
 }
 
+// FP64 arithmetic is what bounds the FP64 applies (a warp's instruction takes
+// about 64 clocks of its quarter of the SM), and away from the liquid all of it
+// multiplies zero weights.  A warp whose row weights (or face coefficients) are
+// all zero therefore writes the zeros without forming them.  0 times an
+// infinity or NaN is not zero, so a tile holding a value of 2^900 or more, an
+// infinity or NaN takes the full arithmetic everywhere (the coefficients are
+// far below 2^100, so nothing else overflows).  FP32 applies are bound by memory
+// and do not test.
+template <class T> __device__ __forceinline__ bool zero_bits(T v) { return v == T(0); }
+template <> __device__ __forceinline__ bool zero_bits<double>(double v) { return (__double_as_longlong(v) << 1) == 0; }
+// d x = x for a diagonal entry d: 1 on an inactive unknown (padding: 0, and x = 0)
+template <class T> __device__ __forceinline__ bool keeps(T d, T x) { return d == T(1) || (d == T(0) && x == T(0)); }
+template <> __device__ __forceinline__ bool keeps<double>(double d, double x) {
+    return __double_as_longlong(d) == 0x3ff0000000000000LL || (zero_bits(d) && zero_bits(x));
+}
+__device__ __forceinline__ bool big_val(double v) { return ((__double2hiint(v) >> 20) & 0x7ff) >= 1023 + 900; }
+__device__ __forceinline__ bool big_val(float) { return false; }
+
 // 2D apply, persistent over the tile list and software-pipelined: while a
 // CTA forms the faces and outputs of one tile, the loads of its next tile are
 // already in flight (registers), and the tile index after that too.  One
@@ -98,6 +116,8 @@ __global__ void __launch_bounds__(256, MINB) k_apply2d(Layout L, const int* __re
     for (; k < ntiles; k += G) {
         const int c0 = (tile % L.ntx) * TX, r0 = (tile / L.ntx) * TY2;
         // 1. stage this tile (p = z + beta p_old in CG mode)
+        constexpr bool SKIP = sizeof(T) == 8;
+        bool big = false;
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int e = t + q * 256;
@@ -115,9 +135,15 @@ __global__ void __launch_bounds__(256, MINB) k_apply2d(Layout L, const int* __re
                     sm.own[1][jj - 1][ii - 1] = v[1];
                     sm.own[2][jj - 1][ii - 1] = v[2];
                 }
-                sm.U[jj][ii] = d.sac[q] * (v[2] - v[0]);
-                sm.V[jj][ii] = d.sac[q] * (v[2] + v[0]);
-                sm.N[jj][ii] = d.san[q] * v[1];
+                const bool far = SKIP && (big_val(v[0]) || big_val(v[1]) || big_val(v[2]));
+                big = big || far;
+                if (!SKIP || __any_sync(__activemask(), far || !zero_bits(d.sac[q]) || !zero_bits(d.san[q]))) {
+                    sm.U[jj][ii] = d.sac[q] * (v[2] - v[0]);
+                    sm.V[jj][ii] = d.sac[q] * (v[2] + v[0]);
+                    sm.N[jj][ii] = d.san[q] * v[1];
+                } else {
+                    sm.U[jj][ii] = sm.V[jj][ii] = sm.N[jj][ii] = T(0);
+                }
             }
         }
         const T ku0 = d.ku[0], ku1 = d.ku[1], kv0 = d.kv[0], kv1 = d.kv[1];
@@ -131,7 +157,8 @@ __global__ void __launch_bounds__(256, MINB) k_apply2d(Layout L, const int* __re
             tile2_load<T, C, MODE>(L, (tile % L.ntx) * TX, (tile / L.ntx) * TY2, cf, x, pold, d);
         }
         (void)tile_cur;
-        __syncthreads();
+        if (SKIP) big = __syncthreads_or(big);
+        else __syncthreads();
         // 3. face values z_f = K_f (B^T x)_f
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
@@ -139,8 +166,12 @@ __global__ void __launch_bounds__(256, MINB) k_apply2d(Layout L, const int* __re
             if (e < FC2) {
                 const int jj = e / (TX + 1), ii = e - jj * (TX + 1);
                 const T ku = q == 0 ? ku0 : ku1, kv = q == 0 ? kv0 : kv1;
-                sm.Zu[jj][ii] = ku * ((sm.U[jj][ii + 1] - sm.U[jj][ii]) + (sm.N[jj][ii + 1] - sm.N[jj + 1][ii + 1]));
-                sm.Zv[jj][ii] = kv * ((sm.V[jj + 1][ii] - sm.V[jj][ii]) + (sm.N[jj + 1][ii] - sm.N[jj + 1][ii + 1]));
+                if (!SKIP || big || __any_sync(__activemask(), !zero_bits(ku) || !zero_bits(kv))) {
+                    sm.Zu[jj][ii] = ku * ((sm.U[jj][ii + 1] - sm.U[jj][ii]) + (sm.N[jj][ii + 1] - sm.N[jj + 1][ii + 1]));
+                    sm.Zv[jj][ii] = kv * ((sm.V[jj + 1][ii] - sm.V[jj][ii]) + (sm.N[jj + 1][ii] - sm.N[jj + 1][ii + 1]));
+                } else {
+                    sm.Zu[jj][ii] = sm.Zv[jj][ii] = T(0);
+                }
             }
         }
         __syncthreads();
@@ -149,23 +180,28 @@ __global__ void __launch_bounds__(256, MINB) k_apply2d(Layout L, const int* __re
             const int tx = t & (TX - 1), ty = t / TX;
             const int64_t o = L.off(c0 + tx, r0 + ty, 0);
             const T txx = sm.own[0][ty][tx], txy = sm.own[1][ty][tx], p_ = sm.own[2][ty][tx];
-            const T zu = sm.Zu[ty + 1][tx], zur = sm.Zu[ty + 1][tx + 1], zud = sm.Zu[ty][tx];
-            const T zv = sm.Zv[ty][tx + 1], zvu = sm.Zv[ty + 1][tx + 1], zvl = sm.Zv[ty][tx];
-            T yp, yxx;
-            if (ac != T(0)) {
-                yp = ac * ((zu - zur) + (zv - zvu));
-                yxx = dc * txx + ac * ((zur - zu) + (zv - zvu));
-            } else {
-                yp = p_;
-                yxx = txx;
+            T yp = p_, yxx = txx, yxy = txy;
+            // (an inactive unknown's row is the identity: weight 0, diagonal 1)
+            if (!SKIP || big || __any_sync(0xffffffffu, !zero_bits(ac) || !zero_bits(an) || !keeps(dn, txy))) {
+                const T zu = sm.Zu[ty + 1][tx], zur = sm.Zu[ty + 1][tx + 1], zud = sm.Zu[ty][tx];
+                const T zv = sm.Zv[ty][tx + 1], zvu = sm.Zv[ty + 1][tx + 1], zvl = sm.Zv[ty][tx];
+                if (ac != T(0)) {
+                    yp = ac * ((zu - zur) + (zv - zvu));
+                    yxx = dc * txx + ac * ((zur - zu) + (zv - zvu));
+                }
+                yxy = dn * txy + an * ((zu - zud) + (zv - zvl));
             }
-            T yxy = dn * txy + an * ((zu - zud) + (zv - zvl));
             if (MODE == MODE_RESID) {
                 yxx = b[o] - yxx; yxy = b[S + o] - yxy; yp = b[2 * S + o] - yp;
             }
             y[o] = yxx; y[S + o] = yxy; y[2 * S + o] = yp;
             if (MODE == MODE_RESID) { acc.add(yxx, yxx); acc.add(yxy, yxy); acc.add(yp, yp); }
-            else if (MODE == MODE_CG) { acc.add(txx, yxx); acc.add(txy, yxy); acc.add(p_, yp); }
+            else if (MODE == MODE_CG) {
+                // (zeros add nothing)
+                if (!SKIP || __any_sync(0xffffffffu, !zero_bits(txx) || !zero_bits(txy) || !zero_bits(p_))) {
+                    acc.add(txx, yxx); acc.add(txy, yxy); acc.add(p_, yp);
+                }
+            }
         }
         __syncthreads();                         // the next tile's staging reuses shared memory
     }
@@ -619,6 +655,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
     // the padded rows (row R is the next plane's pad row; later rows are only
     // read for the outputs and faces of inactive tile rows past the grid)
     // are zero, so every read stays inside the guards.
+    constexpr bool SKIP = sizeof(T) == 8;         // warps of zero weights do no arithmetic (see big_val)
+    bool big = false;                             // this thread staged a value too large for that
     auto stage = [&](int q) {
         T(*st)[SM::NS] = sm.st[q & 1];
         const bool own_plane = q >= q0 && q < q0 + zt * TZ3;
@@ -645,12 +683,25 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
             } else {
                 ac = ld<T, C>(a_c, o); axy = ld<T, C>(a_xy, o); axz = ld<T, C>(a_xz, o); ayz = ld<T, C>(a_yz, o);
             }
-            st[0][e] = ac * (v[5] - v[0]);
-            st[1][e] = ac * (v[5] - v[1]);
-            st[2][e] = ac * (v[5] + v[0] + v[1]);
-            st[3][e] = axy * v[2];
-            st[4][e] = axz * v[3];
-            st[5][e] = ayz * v[4];
+            bool work = true;
+            if (SKIP) {
+                bool far = false;
+#pragma unroll
+                for (int f = 0; f < 6; ++f) far = far || big_val(v[f]);
+                big = big || far;
+                work = __any_sync(__activemask(), far || !zero_bits(ac) || !zero_bits(axy) || !zero_bits(axz) || !zero_bits(ayz));
+            }
+            if (work) {
+                st[0][e] = ac * (v[5] - v[0]);
+                st[1][e] = ac * (v[5] - v[1]);
+                st[2][e] = ac * (v[5] + v[0] + v[1]);
+                st[3][e] = axy * v[2];
+                st[4][e] = axz * v[3];
+                st[5][e] = ayz * v[4];
+            } else {
+#pragma unroll
+                for (int f = 0; f < 6; ++f) st[f][e] = T(0);
+            }
         }
     };
     // face coefficients of z_u(q), z_v(q), z_w(q+1) at face position e (zero
@@ -672,7 +723,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
         }
     };
     // z_u(q), z_v(q) from staged planes q and q+1; z_w(q+1) from planes q and q+1
-    auto faces = [&](int q, const T (&k)[FPT][3]) {
+    auto faces = [&](int q, const T (&k)[FPT][3], bool any_big) {
         const T(*A)[SM::NS] = sm.st[q & 1];
         const T(*B)[SM::NS] = sm.st[(q + 1) & 1];
 #pragma unroll
@@ -681,6 +732,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
             if (e >= SM::NF) break;
             const int ii = e % SM::FX, jj = e / SM::FX;
             if (r0 + jj > L.R) {
+                sm.fz[0][q & 1][e] = sm.fz[1][q & 1][e] = sm.fz[2][(q + 1) & 1][e] = T(0);
+                continue;
+            }
+            if (SKIP && !any_big &&
+                !__any_sync(__activemask(), !zero_bits(k[it][0]) || !zero_bits(k[it][1]) || !zero_bits(k[it][2]))) {
                 sm.fz[0][q & 1][e] = sm.fz[1][q & 1][e] = sm.fz[2][(q + 1) & 1][e] = T(0);
                 continue;
             }
@@ -709,21 +765,23 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
     // prologue: planes q0-1 and q0; z_u(q0-1), z_v(q0-1); z_w(q0)
     stage(q0 - 1);
     stage(q0);
-    __syncthreads();
+    if (SKIP) big = __syncthreads_or(big);
+    else __syncthreads();
     T k0[FPT][3];
     face_k(q0 - 1, k0);
-    faces(q0 - 1, k0);
+    faces(q0 - 1, k0, big);
     __syncthreads();
     }
     const int tx = t & (TX - 1), ty = t >> 5;
     auto fi = [](int ii, int jj) { return jj * SM::FX + ii; };
     for (int q = q0; q < q_end; ++q) {
         stage(q + 1);
-        __syncthreads();
+        if (SKIP) big = __syncthreads_or(big);
+        else __syncthreads();
         {
             T kq[FPT][3];
             face_k(q, kq);
-            faces(q, kq);
+            faces(q, kq, big);
         }
         __syncthreads();
         const int r = r0 + ty;
@@ -732,6 +790,22 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
             T v[6];
 #pragma unroll
             for (int f = 0; f < 6; ++f) v[f] = MODE == MODE_CG ? pnew[f * S + o] : x[f * S + o];
+            T ac, axy, axz, ayz, dc, dxy, dxz, dyz;
+            if constexpr (QD) {
+                const uint2 wa = __ldg(qa + o), wd = __ldg(qdg + o);
+                ac = T(plo(wa.x)); axy = T(phi(wa.x)); axz = T(plo(wa.y)); ayz = T(phi(wa.y));
+                dc = T(plo(wd.x)); dxy = T(phi(wd.x)); dxz = T(plo(wd.y)); dyz = T(phi(wd.y));
+            } else {
+                ac = ld<T, C>(a_c, o); axy = ld<T, C>(a_xy, o); axz = ld<T, C>(a_xz, o); ayz = ld<T, C>(a_yz, o);
+                dc = ld<T, C>(d_c, o); dxy = ld<T, C>(d_xy, o); dxz = ld<T, C>(d_xz, o); dyz = ld<T, C>(d_yz, o);
+            }
+            T yv[6];
+#pragma unroll
+            for (int f = 0; f < 6; ++f) yv[f] = v[f];
+            // (an inactive unknown's row is the identity: weight 0, diagonal 1)
+            if (!SKIP || big || __any_sync(__activemask(), !zero_bits(ac) || !zero_bits(axy) || !zero_bits(axz) ||
+                                                               !zero_bits(ayz) || !keeps(dxy, v[2]) || !keeps(dxz, v[3]) ||
+                                                               !keeps(dyz, v[4]))) {
             const T* zu_q = sm.fz[0][q & 1];
             const T* zu_m = sm.fz[0][(q - 1) & 1];
             const T* zv_q = sm.fz[1][q & 1];
@@ -745,27 +819,16 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
             const T zv_cm = zv_q[fi(tx, ty)], zv_qm = zv_m[fi(tx + 1, ty)];
             const T zw = zw_q[fi(tx + 1, ty + 1)], zw_qp = zw_p[fi(tx + 1, ty + 1)];
             const T zw_cm = zw_q[fi(tx, ty + 1)], zw_rm = zw_q[fi(tx + 1, ty)];
-            T ac, axy, axz, ayz, dc, dxy, dxz, dyz;
-            if constexpr (QD) {
-                const uint2 wa = __ldg(qa + o), wd = __ldg(qdg + o);
-                ac = T(plo(wa.x)); axy = T(phi(wa.x)); axz = T(plo(wa.y)); ayz = T(phi(wa.y));
-                dc = T(plo(wd.x)); dxy = T(phi(wd.x)); dxz = T(plo(wd.y)); dyz = T(phi(wd.y));
-            } else {
-                ac = ld<T, C>(a_c, o); axy = ld<T, C>(a_xy, o); axz = ld<T, C>(a_xz, o); ayz = ld<T, C>(a_yz, o);
-                dc = ld<T, C>(d_c, o); dxy = ld<T, C>(d_xy, o); dxz = ld<T, C>(d_xz, o); dyz = ld<T, C>(d_yz, o);
-            }
-            T yv[6];
             if (ac != T(0)) {
                 const T ww = zw - zw_qp;
                 yv[5] = ac * ((zu - zu_cp) + (zv - zv_rp) + ww);
                 yv[0] = dc * (v[0] + T(0.5) * v[1]) + ac * ((zu_cp - zu) + ww);
                 yv[1] = dc * (v[1] + T(0.5) * v[0]) + ac * ((zv_rp - zv) + ww);
-            } else {
-                yv[5] = v[5]; yv[0] = v[0]; yv[1] = v[1];
             }
             yv[2] = dxy * v[2] + axy * ((zu - zu_rm) + (zv - zv_cm));
             yv[3] = dxz * v[3] + axz * ((zu - zu_qm) + (zw - zw_cm));
             yv[4] = dyz * v[4] + ayz * ((zv - zv_qm) + (zw - zw_rm));
+            }
             if (MODE == MODE_RESID) {
                 const T* b = (const T*)args.b;
 #pragma unroll
@@ -777,8 +840,12 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
 #pragma unroll
                 for (int f = 0; f < 6; ++f) acc.add(yv[f], yv[f]);
             } else if (MODE == MODE_CG) {
+                bool some = !SKIP;                // (zeros add nothing)
 #pragma unroll
-                for (int f = 0; f < 6; ++f) acc.add(v[f], yv[f]);
+                for (int f = 0; f < 6; ++f) some = some || !zero_bits(v[f]);
+                if (!SKIP || __any_sync(__activemask(), some))
+#pragma unroll
+                    for (int f = 0; f < 6; ++f) acc.add(v[f], yv[f]);
             }
         }
         // the next step's staging overwrites the staged plane q (read by the

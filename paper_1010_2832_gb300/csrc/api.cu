@@ -315,6 +315,7 @@ stokes_status stokes_apply(stokes_ctx h, const void* x, void* y, int precision) 
     if (!x || !y || x == y) { c.err = "x and y must be distinct non-null device vectors"; return STOKES_ERR_ARG; }
     if (!c.have_weights) { c.err = "stokes_build_weights has not run"; return STOKES_ERR_STATE; }
     ApplyArgs a{};
+    a.tflag = c.A.tile_flag;
     cudaError_t e;
     API_CHECK_CUDA(h, cudaEventRecord(c.ev[0], c.stream));
     // every tile: inactive unknowns outside active tiles must also map x -> x

@@ -40,9 +40,21 @@ constexpr int FC2 = (TY2 + 1) * (TX + 1);     // faces of each direction (297)
 
 template <class T, class C, int MODE>
 __device__ __forceinline__ void tile2_load(const Layout& L, int c0, int r0, const Coef<C>& cf, const T* __restrict__ x,
-                                           const T* __restrict__ pold, Tile2Loads<T>& d) {
+                                           const T* __restrict__ pold, Tile2Loads<T>& d, bool coefs = true) {
     const int t = threadIdx.x;
     const int64_t S = L.stride;
+    if (!coefs) {                                // the staged unknowns alone
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int e = t + q * 256;
+            if (e < ST2) {
+                const int jj = e / (TX + 2), ii = e - jj * (TX + 2);
+#pragma unroll
+                for (int f = 0; f < 3; ++f) d.sx[q][f] = __ldg(x + f * S + L.off(c0 - 1 + ii, r0 - 1 + jj, 0));
+            }
+        }
+        return;
+    }
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
         const int e = t + q * 256;
@@ -71,20 +83,15 @@ __device__ __forceinline__ void tile2_load(const Layout& L, int c0, int r0, cons
 }
 
 // FP64 arithmetic is what bounds the FP64 applies (a warp's instruction takes
-// about 64 clocks of its quarter of the SM), and away from the liquid all of it
-// multiplies zero weights.  A warp whose row weights (or face coefficients) are
-// all zero therefore writes the zeros without forming them.  0 times an
-// infinity or NaN is not zero, so a tile holding a value of 2^900 or more, an
-// infinity or NaN takes the full arithmetic everywhere (the coefficients are
-// far below 2^100, so nothing else overflows).  FP32 applies are bound by memory
-// and do not test.
-template <class T> __device__ __forceinline__ bool zero_bits(T v) { return v == T(0); }
-template <> __device__ __forceinline__ bool zero_bits<double>(double v) { return (__double_as_longlong(v) << 1) == 0; }
-// d x = x for a diagonal entry d: 1 on an inactive unknown (padding: 0, and x = 0)
-template <class T> __device__ __forceinline__ bool keeps(T d, T x) { return d == T(1) || (d == T(0) && x == T(0)); }
-template <> __device__ __forceinline__ bool keeps<double>(double d, double x) {
-    return __double_as_longlong(d) == 0x3ff0000000000000LL || (zero_bits(d) && zero_bits(x));
-}
+// about 64 clocks of its quarter of the SM), and where no unknown is active all
+// of it multiplies zero weights and the operator is the identity.  An apply over
+// the whole grid (PLAIN) therefore copies the tiles (3D: the layers of a unit)
+// without an active unknown and does not read their coefficients.  0 times an
+// infinity or NaN is not zero, so a tile that holds, or borders on, a value of
+// 2^900 or more, an infinity or NaN takes the full arithmetic (the coefficients
+// are far below 2^100, so nothing else overflows).  (Testing the weights warp by
+// warp instead cost full boxes a quarter more: the votes and branches between
+// the FP64 instructions leave the slow pipe idle.)
 __device__ __forceinline__ bool big_val(double v) { return ((__double2hiint(v) >> 20) & 0x7ff) >= 1023 + 900; }
 __device__ __forceinline__ bool big_val(float) { return false; }
 
@@ -107,17 +114,54 @@ __global__ void __launch_bounds__(256, MINB) k_apply2d(Layout L, const int* __re
     const int t = threadIdx.x;
     const int G = gridDim.x;
     auto tile_at = [&](int k) { return tiles ? tiles[k] : k; };
+    constexpr bool SKIP = sizeof(T) == 8 && MODE == MODE_PLAIN;
+    const uint8_t* __restrict__ flags = SKIP ? args.tflag : nullptr;
+    auto active_at = [&](int tile) { return !SKIP || !flags || flags[tile]; };
     Acc<T> acc;
     int k = blockIdx.x;
     Tile2Loads<T> d;
     int tile = k < ntiles ? tile_at(k) : 0;
     int tile_next = k + G < ntiles ? tile_at(k + G) : 0;
+    // (the first tile's loads do not wait for its flag)
+    bool act = active_at(tile), act_next = active_at(tile_next);
     if (k < ntiles) tile2_load<T, C, MODE>(L, (tile % L.ntx) * TX, (tile / L.ntx) * TY2, cf, x, pold, d);
     for (; k < ntiles; k += G) {
         const int c0 = (tile % L.ntx) * TX, r0 = (tile / L.ntx) * TY2;
+        if (SKIP && !act) {
+            T own[2][3];
+            bool big = false;
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                if (t + q * 256 < ST2)
+#pragma unroll
+                    for (int f = 0; f < 3; ++f) {
+                        own[q][f] = d.sx[q][f];
+                        big = big || big_val(own[q][f]);
+                    }
+            if (!__syncthreads_or(big)) {
+                const int kn = k + G;
+                tile = tile_next;
+                act = act_next;
+                if (kn < ntiles) {
+                    tile_next = kn + G < ntiles ? tile_at(kn + G) : 0;
+                    act_next = active_at(tile_next);
+                    tile2_load<T, C, MODE>(L, (tile % L.ntx) * TX, (tile / L.ntx) * TY2, cf, x, pold, d, act);
+                }
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const int e = t + q * 256;
+                    const int jj = e / (TX + 2), ii = e - jj * (TX + 2);
+                    if (e < ST2 && ii >= 1 && ii <= TX && jj >= 1 && jj <= TY2) {
+                        const int64_t o = L.off(c0 - 1 + ii, r0 - 1 + jj, 0);
+#pragma unroll
+                        for (int f = 0; f < 3; ++f) y[f * S + o] = own[q][f];
+                    }
+                }
+                continue;
+            }
+            tile2_load<T, C, MODE>(L, c0, r0, cf, x, pold, d);
+        }
         // 1. stage this tile (p = z + beta p_old in CG mode)
-        constexpr bool SKIP = sizeof(T) == 8;
-        bool big = false;
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int e = t + q * 256;
@@ -135,15 +179,9 @@ __global__ void __launch_bounds__(256, MINB) k_apply2d(Layout L, const int* __re
                     sm.own[1][jj - 1][ii - 1] = v[1];
                     sm.own[2][jj - 1][ii - 1] = v[2];
                 }
-                const bool far = SKIP && (big_val(v[0]) || big_val(v[1]) || big_val(v[2]));
-                big = big || far;
-                if (!SKIP || __any_sync(__activemask(), far || !zero_bits(d.sac[q]) || !zero_bits(d.san[q]))) {
-                    sm.U[jj][ii] = d.sac[q] * (v[2] - v[0]);
-                    sm.V[jj][ii] = d.sac[q] * (v[2] + v[0]);
-                    sm.N[jj][ii] = d.san[q] * v[1];
-                } else {
-                    sm.U[jj][ii] = sm.V[jj][ii] = sm.N[jj][ii] = T(0);
-                }
+                sm.U[jj][ii] = d.sac[q] * (v[2] - v[0]);
+                sm.V[jj][ii] = d.sac[q] * (v[2] + v[0]);
+                sm.N[jj][ii] = d.san[q] * v[1];
             }
         }
         const T ku0 = d.ku[0], ku1 = d.ku[1], kv0 = d.kv[0], kv1 = d.kv[1];
@@ -152,13 +190,14 @@ __global__ void __launch_bounds__(256, MINB) k_apply2d(Layout L, const int* __re
         const int kn = k + G;
         const int tile_cur = tile;
         tile = tile_next;
+        act = act_next;
         if (kn < ntiles) {
             tile_next = kn + G < ntiles ? tile_at(kn + G) : 0;
-            tile2_load<T, C, MODE>(L, (tile % L.ntx) * TX, (tile / L.ntx) * TY2, cf, x, pold, d);
+            act_next = active_at(tile_next);
+            tile2_load<T, C, MODE>(L, (tile % L.ntx) * TX, (tile / L.ntx) * TY2, cf, x, pold, d, act);
         }
         (void)tile_cur;
-        if (SKIP) big = __syncthreads_or(big);
-        else __syncthreads();
+        __syncthreads();
         // 3. face values z_f = K_f (B^T x)_f
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
@@ -166,12 +205,8 @@ __global__ void __launch_bounds__(256, MINB) k_apply2d(Layout L, const int* __re
             if (e < FC2) {
                 const int jj = e / (TX + 1), ii = e - jj * (TX + 1);
                 const T ku = q == 0 ? ku0 : ku1, kv = q == 0 ? kv0 : kv1;
-                if (!SKIP || big || __any_sync(__activemask(), !zero_bits(ku) || !zero_bits(kv))) {
-                    sm.Zu[jj][ii] = ku * ((sm.U[jj][ii + 1] - sm.U[jj][ii]) + (sm.N[jj][ii + 1] - sm.N[jj + 1][ii + 1]));
-                    sm.Zv[jj][ii] = kv * ((sm.V[jj + 1][ii] - sm.V[jj][ii]) + (sm.N[jj + 1][ii] - sm.N[jj + 1][ii + 1]));
-                } else {
-                    sm.Zu[jj][ii] = sm.Zv[jj][ii] = T(0);
-                }
+                sm.Zu[jj][ii] = ku * ((sm.U[jj][ii + 1] - sm.U[jj][ii]) + (sm.N[jj][ii + 1] - sm.N[jj + 1][ii + 1]));
+                sm.Zv[jj][ii] = kv * ((sm.V[jj + 1][ii] - sm.V[jj][ii]) + (sm.N[jj + 1][ii] - sm.N[jj + 1][ii + 1]));
             }
         }
         __syncthreads();
@@ -180,28 +215,23 @@ __global__ void __launch_bounds__(256, MINB) k_apply2d(Layout L, const int* __re
             const int tx = t & (TX - 1), ty = t / TX;
             const int64_t o = L.off(c0 + tx, r0 + ty, 0);
             const T txx = sm.own[0][ty][tx], txy = sm.own[1][ty][tx], p_ = sm.own[2][ty][tx];
-            T yp = p_, yxx = txx, yxy = txy;
-            // (an inactive unknown's row is the identity: weight 0, diagonal 1)
-            if (!SKIP || big || __any_sync(0xffffffffu, !zero_bits(ac) || !zero_bits(an) || !keeps(dn, txy))) {
-                const T zu = sm.Zu[ty + 1][tx], zur = sm.Zu[ty + 1][tx + 1], zud = sm.Zu[ty][tx];
-                const T zv = sm.Zv[ty][tx + 1], zvu = sm.Zv[ty + 1][tx + 1], zvl = sm.Zv[ty][tx];
-                if (ac != T(0)) {
-                    yp = ac * ((zu - zur) + (zv - zvu));
-                    yxx = dc * txx + ac * ((zur - zu) + (zv - zvu));
-                }
-                yxy = dn * txy + an * ((zu - zud) + (zv - zvl));
+            const T zu = sm.Zu[ty + 1][tx], zur = sm.Zu[ty + 1][tx + 1], zud = sm.Zu[ty][tx];
+            const T zv = sm.Zv[ty][tx + 1], zvu = sm.Zv[ty + 1][tx + 1], zvl = sm.Zv[ty][tx];
+            T yp, yxx;
+            if (ac != T(0)) {
+                yp = ac * ((zu - zur) + (zv - zvu));
+                yxx = dc * txx + ac * ((zur - zu) + (zv - zvu));
+            } else {
+                yp = p_;
+                yxx = txx;
             }
+            T yxy = dn * txy + an * ((zu - zud) + (zv - zvl));
             if (MODE == MODE_RESID) {
                 yxx = b[o] - yxx; yxy = b[S + o] - yxy; yp = b[2 * S + o] - yp;
             }
             y[o] = yxx; y[S + o] = yxy; y[2 * S + o] = yp;
             if (MODE == MODE_RESID) { acc.add(yxx, yxx); acc.add(yxy, yxy); acc.add(yp, yp); }
-            else if (MODE == MODE_CG) {
-                // (zeros add nothing)
-                if (!SKIP || __any_sync(0xffffffffu, !zero_bits(txx) || !zero_bits(txy) || !zero_bits(p_))) {
-                    acc.add(txx, yxx); acc.add(txy, yxy); acc.add(p_, yp);
-                }
-            }
+            else if (MODE == MODE_CG) { acc.add(txx, yxx); acc.add(txy, yxy); acc.add(p_, yp); }
         }
         __syncthreads();                         // the next tile's staging reuses shared memory
     }
@@ -628,6 +658,19 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
             for (int dy = 0; dy < 2; ++dy)
                 if (2 * uy + dy < L.nty && zt * uz + dz < L.ntz) mask |= 1u << (dy + 2 * dz);
     }
+    // PLAIN FP64: the unit's layers that hold an active unknown (bit dz); the
+    // others are copied unless a value is too large for that (see big_val)
+    constexpr bool SKIP = sizeof(T) == 8 && MODE == MODE_PLAIN;
+    unsigned lay = 0xfu;
+    if (SKIP && args.tflag) {
+        lay = 0;
+        for (int dz = 0; dz < zt; ++dz)
+            if (!((mask >> (2 * dz)) & 3u)) lay |= 1u << dz;         // past the grid: never reached
+        for (int dz = 0; dz < zt; ++dz)
+            for (int dy = 0; dy < 2; ++dy)
+                if (((mask >> (dy + 2 * dz)) & 1u) && args.tflag[((int64_t)(zt * uz + dz) * L.nty + 2 * uy + dy) * L.ntx + ux])
+                    lay |= 1u << dz;
+    }
     const int c0 = ux * TX, r0 = uy * UY3, q0 = uz * zt * TZ3;
     const int64_t S = L.stride;
     const C *a_c = cf.f[0], *a_xy = cf.f[1], *a_xz = cf.f[2], *a_yz = cf.f[3];
@@ -655,8 +698,6 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
     // the padded rows (row R is the next plane's pad row; later rows are only
     // read for the outputs and faces of inactive tile rows past the grid)
     // are zero, so every read stays inside the guards.
-    constexpr bool SKIP = sizeof(T) == 8;         // warps of zero weights do no arithmetic (see big_val)
-    bool big = false;                             // this thread staged a value too large for that
     auto stage = [&](int q) {
         T(*st)[SM::NS] = sm.st[q & 1];
         const bool own_plane = q >= q0 && q < q0 + zt * TZ3;
@@ -683,25 +724,12 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
             } else {
                 ac = ld<T, C>(a_c, o); axy = ld<T, C>(a_xy, o); axz = ld<T, C>(a_xz, o); ayz = ld<T, C>(a_yz, o);
             }
-            bool work = true;
-            if (SKIP) {
-                bool far = false;
-#pragma unroll
-                for (int f = 0; f < 6; ++f) far = far || big_val(v[f]);
-                big = big || far;
-                work = __any_sync(__activemask(), far || !zero_bits(ac) || !zero_bits(axy) || !zero_bits(axz) || !zero_bits(ayz));
-            }
-            if (work) {
-                st[0][e] = ac * (v[5] - v[0]);
-                st[1][e] = ac * (v[5] - v[1]);
-                st[2][e] = ac * (v[5] + v[0] + v[1]);
-                st[3][e] = axy * v[2];
-                st[4][e] = axz * v[3];
-                st[5][e] = ayz * v[4];
-            } else {
-#pragma unroll
-                for (int f = 0; f < 6; ++f) st[f][e] = T(0);
-            }
+            st[0][e] = ac * (v[5] - v[0]);
+            st[1][e] = ac * (v[5] - v[1]);
+            st[2][e] = ac * (v[5] + v[0] + v[1]);
+            st[3][e] = axy * v[2];
+            st[4][e] = axz * v[3];
+            st[5][e] = ayz * v[4];
         }
     };
     // face coefficients of z_u(q), z_v(q), z_w(q+1) at face position e (zero
@@ -723,7 +751,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
         }
     };
     // z_u(q), z_v(q) from staged planes q and q+1; z_w(q+1) from planes q and q+1
-    auto faces = [&](int q, const T (&k)[FPT][3], bool any_big) {
+    auto faces = [&](int q, const T (&k)[FPT][3]) {
         const T(*A)[SM::NS] = sm.st[q & 1];
         const T(*B)[SM::NS] = sm.st[(q + 1) & 1];
 #pragma unroll
@@ -732,11 +760,6 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
             if (e >= SM::NF) break;
             const int ii = e % SM::FX, jj = e / SM::FX;
             if (r0 + jj > L.R) {
-                sm.fz[0][q & 1][e] = sm.fz[1][q & 1][e] = sm.fz[2][(q + 1) & 1][e] = T(0);
-                continue;
-            }
-            if (SKIP && !any_big &&
-                !__any_sync(__activemask(), !zero_bits(k[it][0]) || !zero_bits(k[it][1]) || !zero_bits(k[it][2]))) {
                 sm.fz[0][q & 1][e] = sm.fz[1][q & 1][e] = sm.fz[2][(q + 1) & 1][e] = T(0);
                 continue;
             }
@@ -761,27 +784,67 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
     for (int dz = 0; dz < zt; ++dz)
         if ((mask >> (2 * dz)) & 3u) dz_end = dz + 1;
     const int q_end = q0 + TZ3 * dz_end;
-    if (q_end > q0) {
+    auto act_plane = [&](int q) { return q >= q0 && q < q_end && ((lay >> ((q - q0) / TZ3)) & 1u); };
+    auto plane_big = [&](int q) -> bool {          // this thread's part of plane q with its halo
+        bool big = false;
+        for (int e = t; e < SM::NS; e += 256) {
+            const int ii = e % SM::SX, jj = e / SM::SX;
+            if (r0 - 1 + jj > L.R) continue;
+            const int64_t o = L.off(c0 - 1 + ii, r0 - 1 + jj, q);
+#pragma unroll
+            for (int f = 0; f < 6; ++f) big = big || big_val(x[f * S + o]);
+        }
+        return big;
+    };
+    if constexpr (SKIP) {
+        if (lay != 0xfu) {
+            // the copied planes and their neighbours, before anything is written
+            auto copied = [&](int q) { return q >= q0 && q < q_end && !act_plane(q); };
+            bool big = false;
+            for (int q = q0 - 1; q <= q_end; ++q)
+                if (copied(q - 1) || copied(q) || copied(q + 1)) big = plane_big(q) || big;
+            if (__syncthreads_or(big)) lay = 0xfu;
+        }
+    }
+    if (q_end > q0 && (!SKIP || act_plane(q0))) {
     // prologue: planes q0-1 and q0; z_u(q0-1), z_v(q0-1); z_w(q0)
     stage(q0 - 1);
     stage(q0);
-    if (SKIP) big = __syncthreads_or(big);
-    else __syncthreads();
+    __syncthreads();
     T k0[FPT][3];
     face_k(q0 - 1, k0);
-    faces(q0 - 1, k0, big);
+    faces(q0 - 1, k0);
     __syncthreads();
     }
     const int tx = t & (TX - 1), ty = t >> 5;
     auto fi = [](int ii, int jj) { return jj * SM::FX + ii; };
     for (int q = q0; q < q_end; ++q) {
+        if (SKIP && !act_plane(q)) {
+            // a copied plane; what the planes after it need: the staged planes
+            // q, q + 1 and the faces of q
+            if (act_plane(q + 1)) {
+                stage(q);
+                stage(q + 1);
+                __syncthreads();
+                T kq[FPT][3];
+                face_k(q, kq);
+                faces(q, kq);
+                __syncthreads();
+            }
+            const int r = r0 + ty;
+            if (active(r, q)) {
+                const int64_t o = L.off(c0 + tx, r, q);
+#pragma unroll
+                for (int f = 0; f < 6; ++f) y[f * S + o] = x[f * S + o];
+            }
+            continue;
+        }
         stage(q + 1);
-        if (SKIP) big = __syncthreads_or(big);
-        else __syncthreads();
+        __syncthreads();
         {
             T kq[FPT][3];
             face_k(q, kq);
-            faces(q, kq, big);
+            faces(q, kq);
         }
         __syncthreads();
         const int r = r0 + ty;
@@ -790,22 +853,6 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
             T v[6];
 #pragma unroll
             for (int f = 0; f < 6; ++f) v[f] = MODE == MODE_CG ? pnew[f * S + o] : x[f * S + o];
-            T ac, axy, axz, ayz, dc, dxy, dxz, dyz;
-            if constexpr (QD) {
-                const uint2 wa = __ldg(qa + o), wd = __ldg(qdg + o);
-                ac = T(plo(wa.x)); axy = T(phi(wa.x)); axz = T(plo(wa.y)); ayz = T(phi(wa.y));
-                dc = T(plo(wd.x)); dxy = T(phi(wd.x)); dxz = T(plo(wd.y)); dyz = T(phi(wd.y));
-            } else {
-                ac = ld<T, C>(a_c, o); axy = ld<T, C>(a_xy, o); axz = ld<T, C>(a_xz, o); ayz = ld<T, C>(a_yz, o);
-                dc = ld<T, C>(d_c, o); dxy = ld<T, C>(d_xy, o); dxz = ld<T, C>(d_xz, o); dyz = ld<T, C>(d_yz, o);
-            }
-            T yv[6];
-#pragma unroll
-            for (int f = 0; f < 6; ++f) yv[f] = v[f];
-            // (an inactive unknown's row is the identity: weight 0, diagonal 1)
-            if (!SKIP || big || __any_sync(__activemask(), !zero_bits(ac) || !zero_bits(axy) || !zero_bits(axz) ||
-                                                               !zero_bits(ayz) || !keeps(dxy, v[2]) || !keeps(dxz, v[3]) ||
-                                                               !keeps(dyz, v[4]))) {
             const T* zu_q = sm.fz[0][q & 1];
             const T* zu_m = sm.fz[0][(q - 1) & 1];
             const T* zv_q = sm.fz[1][q & 1];
@@ -819,16 +866,27 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
             const T zv_cm = zv_q[fi(tx, ty)], zv_qm = zv_m[fi(tx + 1, ty)];
             const T zw = zw_q[fi(tx + 1, ty + 1)], zw_qp = zw_p[fi(tx + 1, ty + 1)];
             const T zw_cm = zw_q[fi(tx, ty + 1)], zw_rm = zw_q[fi(tx + 1, ty)];
+            T ac, axy, axz, ayz, dc, dxy, dxz, dyz;
+            if constexpr (QD) {
+                const uint2 wa = __ldg(qa + o), wd = __ldg(qdg + o);
+                ac = T(plo(wa.x)); axy = T(phi(wa.x)); axz = T(plo(wa.y)); ayz = T(phi(wa.y));
+                dc = T(plo(wd.x)); dxy = T(phi(wd.x)); dxz = T(plo(wd.y)); dyz = T(phi(wd.y));
+            } else {
+                ac = ld<T, C>(a_c, o); axy = ld<T, C>(a_xy, o); axz = ld<T, C>(a_xz, o); ayz = ld<T, C>(a_yz, o);
+                dc = ld<T, C>(d_c, o); dxy = ld<T, C>(d_xy, o); dxz = ld<T, C>(d_xz, o); dyz = ld<T, C>(d_yz, o);
+            }
+            T yv[6];
             if (ac != T(0)) {
                 const T ww = zw - zw_qp;
                 yv[5] = ac * ((zu - zu_cp) + (zv - zv_rp) + ww);
                 yv[0] = dc * (v[0] + T(0.5) * v[1]) + ac * ((zu_cp - zu) + ww);
                 yv[1] = dc * (v[1] + T(0.5) * v[0]) + ac * ((zv_rp - zv) + ww);
+            } else {
+                yv[5] = v[5]; yv[0] = v[0]; yv[1] = v[1];
             }
             yv[2] = dxy * v[2] + axy * ((zu - zu_rm) + (zv - zv_cm));
             yv[3] = dxz * v[3] + axz * ((zu - zu_qm) + (zw - zw_cm));
             yv[4] = dyz * v[4] + ayz * ((zv - zv_qm) + (zw - zw_rm));
-            }
             if (MODE == MODE_RESID) {
                 const T* b = (const T*)args.b;
 #pragma unroll
@@ -840,12 +898,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
 #pragma unroll
                 for (int f = 0; f < 6; ++f) acc.add(yv[f], yv[f]);
             } else if (MODE == MODE_CG) {
-                bool some = !SKIP;                // (zeros add nothing)
 #pragma unroll
-                for (int f = 0; f < 6; ++f) some = some || !zero_bits(v[f]);
-                if (!SKIP || __any_sync(__activemask(), some))
-#pragma unroll
-                    for (int f = 0; f < 6; ++f) acc.add(v[f], yv[f]);
+                for (int f = 0; f < 6; ++f) acc.add(v[f], yv[f]);
             }
         }
         // the next step's staging overwrites the staged plane q (read by the
@@ -888,7 +942,9 @@ static cudaError_t launch_mode(const Layout& L, const int* tiles, int ntiles, co
     static int cache2[16], cache3[16];
     if (L.dim == 2) {
         // FP64 vectors: one slot per thread, software-pipelined over the tiles
-        // (bound by the FP64 pipe; the unconstrained build is faster)
+        // (bound by the FP64 pipe).  In the CG loop the unconstrained build is
+        // faster; over the whole grid, copied tiles included, three CTAs per SM
+        // (1024^2 bumps 26.5 against 28.2 us, 2048^2 box 269 against 273)
         // FP32 vectors: four slots per thread, four tiles per CTA, 16-byte
         // loads and stores of the vectors, which callers' arrays (a view at
         // an odd offset) need not allow: those take one slot per thread
@@ -907,7 +963,7 @@ static cudaError_t launch_mode(const Layout& L, const int* tiles, int ntiles, co
                 k_apply2d<T, C, MODE, MINB><<<grid, 256, 0, s>>>(L, tiles, cf, x, y, a, ntiles);
             }
         } else {
-            constexpr int MINB = 1;
+            constexpr int MINB = MODE == MODE_PLAIN ? 3 : 1;
             const int grid = std::min(ntiles, resident_ctas((const void*)k_apply2d<T, C, MODE, MINB>, 256, 0, cache2));
             k_apply2d<T, C, MODE, MINB><<<grid, 256, 0, s>>>(L, tiles, cf, x, y, a, ntiles);
         }

@@ -79,6 +79,7 @@ struct ApplyArgs {
     const uint8_t* umask;
     int nunits;
     int zt;
+    const uint8_t* tflag;   // PLAIN: tiles holding an active unknown (nullptr: take every tile as one)
 };
 
 struct Ctx;   // defined in api.cu

@@ -1,5 +1,5 @@
-"""The FP64 applies leave out the arithmetic of warps whose weights are all
-zero.  Against the oracle's matrix on geometries with large inactive regions,
+"""The FP64 apply over a whole grid copies tiles (3D: layers of a unit) that
+hold no active unknown.  Against the oracle's matrix on geometries with large inactive regions,
 at sizes around the tiles; and infinities, NaN and values near the overflow
 limit must spread as the full arithmetic spreads them (0 times infinity is NaN),
 which the FP32 apply, without such a shortcut, shows."""
@@ -18,6 +18,7 @@ CASES = {
     "rand2d": lambda: W.random_small((33, 17), seed=5),
     "rand3d": lambda: W.random_small((37, 19, 23), seed=6, dim=3),
     "col3d": lambda: W.column_3d(24),
+    "tall3d": lambda: W.random_small((20, 9, 61), seed=9, dim=3),
 }
 _c = {}
 

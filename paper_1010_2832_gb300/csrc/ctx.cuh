@@ -83,6 +83,7 @@ struct Ctx {
     unsigned* counter = nullptr;
     unsigned long long* gather = nullptr;   // slots of the cooperative CG kernels (grid_gather.cuh)
     unsigned long long* zwords = nullptr;   // 2D: boundary values between their CTAs, allocated on first use
+    unsigned long long* swwords = nullptr;  // the same of the Schwarz form
     CgWork<double> w64;
     CgWork<float> w32;
     double* b64 = nullptr;       // rhs (solve_step)
@@ -149,6 +150,9 @@ cudaError_t launch_apply_mode(const Layout& L, const int* tiles, int ntiles, con
 // small enough (*taken says whether it was launched)
 template <class T, class C>
 cudaError_t launch_cg_loop(Ctx* c, CgWork<T>& w, const T* minv, const Coef<C>& cf, int update_ctas, bool* taken);
+
+// schwarz_loop.cu: the same for the Schwarz-preconditioned loop
+cudaError_t launch_schwarz_loop(Ctx* c, const struct SchwarzPlan& P, int finish_ctas, bool* taken);
 
 }  // namespace stk
 

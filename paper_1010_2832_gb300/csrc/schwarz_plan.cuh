@@ -161,8 +161,7 @@ __device__ __forceinline__ void sw_hl_scale(float m, float& sc, float& inv) {
 // Split of the vector v (n entries, scaled by sc) into FP16 hi + lo parts,
 // one entry per thread (threads 0..111), into hb[0][.] and hb[1][.]; entries
 // from n to 111 are zero.
-__device__ __forceinline__ void sw_split(const float* v, int n, float sc, __half* hb) {
-    const int t = threadIdx.x;
+__device__ __forceinline__ void sw_split(int t, const float* v, int n, float sc, __half* hb) {
     if (t < 16 * 7) {
         const float x = t < n ? v[t] * sc : 0.f;
         const __half hi = __float2half_rn(x);
@@ -176,16 +175,39 @@ __device__ __forceinline__ void sw_split(const float* v, int n, float sc, __half
 // largest magnitudes (one word each).
 constexpr int SW_HB_HALVES = 2 * 16 * 7 + 2 * 16 * 7 + 2 * 4;
 
-// Largest |v[k]| over k < n (up to 128 entries), every thread of warps 0..3
-// taking one entry: a warp reduction, the four warps' results through wm,
-// one barrier (every thread of the CTA must call it).
-__device__ __forceinline__ float sw_cta_absmax(const float* v, int n, unsigned* wm) {
-    const int t = threadIdx.x, warp = t >> 5;
+// The threads that solve a patch: a whole CTA (CtaGroup), or 128 threads of it
+// with a named barrier of their own (BarGroup).
+struct CtaGroup {
+    __device__ __forceinline__ int thread() const { return threadIdx.x; }
+    __device__ __forceinline__ void sync() const { __syncthreads(); }
+};
+struct BarGroup {
+    int t, id;                      // thread within the group; barrier 1..15
+    __device__ __forceinline__ int thread() const { return t; }
+    __device__ __forceinline__ void sync() const { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
+    // barrier, and whether any thread's p is set
+    __device__ __forceinline__ bool any(bool p) const {
+        int r;
+        asm volatile(
+            "{\n .reg .pred p, q;\n setp.ne.b32 p, %1, 0;\n bar.red.or.pred q, %2, 128, p;\n selp.b32 %0, 1, 0, q;\n}"
+            : "=r"(r)
+            : "r"((int)p), "r"(id)
+            : "memory");
+        return r != 0;
+    }
+};
+
+// Largest |v[k]| over k < n (up to 128 entries), every thread of the group's
+// warps 0..3 taking one entry: a warp reduction, the four warps' results
+// through wm, one barrier (every thread of the group must call it).
+template <class G>
+__device__ __forceinline__ float sw_cta_absmax(const G& grp, const float* v, int n, unsigned* wm) {
+    const int t = grp.thread(), warp = t >> 5;
     if (warp < 4) {
         const unsigned m = __reduce_max_sync(0xffffffffu, t < n ? __float_as_uint(fabsf(v[t])) : 0u);
         if ((t & 31) == 0) wm[warp] = m;
     }
-    __syncthreads();
+    grp.sync();
     const uint4 a = *reinterpret_cast<const uint4*>(wm);
     return __uint_as_float(max(max(a.x, a.y), max(a.z, a.w)));
 }
@@ -251,7 +273,7 @@ __device__ __forceinline__ void sw_cols(uint32_t X, int ntile, int lane, const u
 }
 
 // s <- X~^T diag(rho^2) X~ s for the stored factor F of an n-unknown patch in
-// shared memory, by warps 0-3 of the CTA (every thread of the CTA must call
+// shared memory, by warps 0-3 of the group (every thread of the group must call
 // it, with at least 112 threads).  X~ is cut into 16 x 16 tiles (rows and
 // columns up to 112); tiles wholly above the diagonal are skipped and the
 // upper 8 x 8 block of each diagonal tile (not stored: rows of the first
@@ -271,8 +293,9 @@ __device__ __forceinline__ void sw_cols(uint32_t X, int ntile, int lane, const u
 // of scratch and may be s itself (s is not read once split).  Ends after a
 // barrier with z in s[0, n) (entries from n to the last tile's end hold
 // finite values that callers do not read).
-__device__ __forceinline__ void sw_factor_products(const uint8_t* F, int n, float* s, float* y, __half* hb) {
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+template <class G>
+__device__ __forceinline__ void sw_factor_products(const G& grp, const uint8_t* F, int n, float* s, float* y, __half* hb) {
+    const int t = grp.thread(), warp = t >> 5, lane = t & 31;
     const float* rs = reinterpret_cast<const float*>(F);
     const uint32_t X = smem_u32(F + SW_RS_BYTES);
     uint32_t* rowtab = reinterpret_cast<uint32_t*>(hb + 2 * 16 * 7);
@@ -289,9 +312,9 @@ __device__ __forceinline__ void sw_factor_products(const uint8_t* F, int n, floa
         rowtab[t] = (2u * (32u * R * (R + 1u) + (uint32_t)(row & 7) * 8u)) | ((32u * w) << 16);
     }
     float sc, inv;
-    sw_hl_scale(sw_cta_absmax(s, n, wm), sc, inv);
-    sw_split(s, n, sc, hb);
-    __syncthreads();
+    sw_hl_scale(sw_cta_absmax(grp, s, n, wm), sc, inv);
+    sw_split(t, s, n, sc, hb);
+    grp.sync();
     if (warp < 4) {
         float dA[4] = {0.f, 0.f, 0.f, 0.f}, dB[4] = {0.f, 0.f, 0.f, 0.f};
         switch (warp) {
@@ -315,10 +338,10 @@ __device__ __forceinline__ void sw_factor_products(const uint8_t* F, int n, floa
             }
         }
     }
-    __syncthreads();
-    sw_hl_scale(sw_cta_absmax(y, n, wm), sc, inv);
-    sw_split(y, n, sc, hb);          // hb of the first product is no longer read
-    __syncthreads();
+    grp.sync();
+    sw_hl_scale(sw_cta_absmax(grp, y, n, wm), sc, inv);
+    sw_split(t, y, n, sc, hb);          // hb of the first product is no longer read
+    grp.sync();
     if (warp < 4) {
         float dA[4] = {0.f, 0.f, 0.f, 0.f}, dB[4] = {0.f, 0.f, 0.f, 0.f};
         switch (warp) {
@@ -342,7 +365,10 @@ __device__ __forceinline__ void sw_factor_products(const uint8_t* F, int n, floa
             }
         }
     }
-    __syncthreads();
+    grp.sync();
+}
+__device__ __forceinline__ void sw_factor_products(const uint8_t* F, int n, float* s, float* y, __half* hb) {
+    sw_factor_products(CtaGroup(), F, n, s, y, hb);
 }
 
 }  // namespace stk

@@ -1,4 +1,5 @@
-"""The one-kernel CG loop of small 2D systems against the same solve launched
+"""The one-kernel CG loops of small 2D systems (Jacobi, and Schwarz with its
+resident patch factors) against the same solve launched
 kernel by kernel (use_graph = 0): the arithmetic and the order of every sum are
 the same, so iterates, iteration counts and statuses agree bit for bit.  Sizes:
 few CTAs (each forms the totals itself), more than 64 (the reducer CTA), FP64
@@ -56,6 +57,25 @@ def test_loop_matches_separate_kernels(name, mode):
         assert torch.equal(x, x2)
         st3, x3 = _solve(ctx, b, mode=mode, **kw)               # and again on the same context
         assert torch.equal(x, x3) and st3.iterations == st.iterations
+
+
+SCHWARZ = dict(CASES,
+               bumps160=lambda: W.bumps_2d(160, seed=5, rho_split=False),   # two patches per group
+               box96=lambda: W.full_box(96, 2),                             # 625 patches
+               box150=lambda: W.full_box(150, 2),                           # 1,444 patches, three per group
+               strip=lambda: W.random_small((301, 9), seed=4))
+
+
+@pytest.mark.parametrize("name", list(SCHWARZ))
+def test_schwarz_loop_matches_separate_kernels(name):
+    CASES.update(SCHWARZ)
+    ctx, b = _system(name)
+    for kw in (dict(tol=1e-10), dict(tol=1e-8, max_iter=5), dict(tol=1e-30, max_iter=60, max_outer=1, inner_tol=1e-30)):
+        st, x = _solve(ctx, b, mode=1, precond=2, **kw)
+        st2, x2 = _solve(ctx, b, mode=1, precond=2, use_graph=0, check_every=2, **kw)
+        assert (st.status, st.iterations, st.outer) == (st2.status, st2.iterations, st2.outer)
+        assert st.rel_residual == st2.rel_residual
+        assert torch.equal(x, x2)
 
 
 @pytest.mark.parametrize("mode", [0, 1])

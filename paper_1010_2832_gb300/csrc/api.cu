@@ -457,7 +457,7 @@ stokes_status stokes_solve_step(stokes_ctx h, const double* const* u_star, doubl
     double* outs[6];
     for (int f = 0; f < c.nf - 1; ++f) outs[f] = tau_out[f];
     outs[c.nf - 1] = p_out;
-    API_CHECK_CUDA(h, launch_unpack(&c, c.x64, outs, 1));
+    API_CHECK_CUDA(h, launch_unpack(&c, c.x64, outs, 2));
     API_CHECK_CUDA(h, cudaEventRecord(c.ev[3], c.stream));
     API_CHECK_CUDA(h, cudaEventSynchronize(c.ev[3]));
     if (st) {

@@ -720,7 +720,7 @@ static cudaError_t enqueue(stokes_batch b, const stokes_batch_io* io) {
         double* outs[6];
         for (int f = 0; f < c->nf - 1; ++f) outs[f] = io[i].tau_out[f];
         outs[c->nf - 1] = io[i].p_out;
-        launch_unpack(c, c->x64, outs, 1);
+        launch_unpack(c, c->x64, outs, 2);
         c->stream = keep;
     }
     return cudaGetLastError();

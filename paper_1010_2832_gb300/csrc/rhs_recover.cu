@@ -238,19 +238,25 @@ __global__ void k_recover3d(Layout L, DevArrays D, FacePtrs us, const double* x,
     }
 }
 
-// slot field f <-> field-layout array of its site kind
+// slot field f <-> field-layout array of its site kind.  TO_FIELDS 2: a solve's
+// result, 0 where the unknown is not active (the solver writes the slots of
+// active tiles only; the others may hold an earlier geometry's solution).
 struct FieldMap { double* p[6]; };
-__global__ void k_slots_fields(Layout L, const double* src, double* dst, int to_fields, int nf, int64_t f_off0,
-                               FieldMap fm, int copy_mode) {
+template <int TO_FIELDS>
+__global__ void __launch_bounds__(256) k_slots_fields(Layout L, DevArrays D, const double* __restrict__ src,
+                                                      double* __restrict__ dst, int nf, FieldMap fm) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     int j = blockIdx.y * blockDim.y + threadIdx.y;
     int k = blockIdx.z;
     if (i > L.nx || j > L.ny || (L.dim == 3 && k > L.nz)) return;
     int64_t o = L.off(i + 1, j + 1, L.dim == 2 ? 0 : k + 1);
     for (int f = 0; f < nf; ++f) {
-        int kind;
-        if (L.dim == 2) kind = (f == 1) ? 1 : 0;
-        else kind = (f <= 1 || f == 5) ? 0 : (f == 2 ? 4 : f == 3 ? 5 : 6);
+        int kind, site;
+        if (L.dim == 2) kind = site = (f == 1) ? 1 : 0;
+        else {
+            kind = (f <= 1 || f == 5) ? 0 : (f == 2 ? 4 : f == 3 ? 5 : 6);
+            site = (f <= 1 || f == 5) ? 0 : f - 1;
+        }
         bool ex;
         int64_t fi;
         if (L.dim == 2) {
@@ -263,10 +269,11 @@ __global__ void k_slots_fields(Layout L, const double* src, double* dst, int to_
         }
         if (!ex) continue;
         double* fp = fm.p[f];
-        if (to_fields) fp[fi] = src[(int64_t)f * L.stride + o];
-        else dst[(int64_t)f * L.stride + o] = fp[fi];
+        const int64_t of = (int64_t)f * L.stride + o;
+        if (TO_FIELDS == 2) fp[fi] = D.act[site][o] ? src[of] : 0.0;
+        else if (TO_FIELDS) fp[fi] = src[of];
+        else dst[of] = fp[fi];
     }
-    (void)f_off0; (void)copy_mode;
 }
 
 static dim3 slot_grid(const Layout& L) {
@@ -297,7 +304,8 @@ cudaError_t launch_recover(Ctx* c, const double* const* ustar, const double* x, 
     return cudaGetLastError();
 }
 
-// Unknown vector <-> separate field-layout arrays (one per unknown field).
+// Unknown vector <-> separate field-layout arrays (one per unknown field);
+// to_fields 2: 0 on inactive unknowns.
 cudaError_t launch_unpack(Ctx* c, const double* slots, double* const* fields, int to_fields) {
     const Layout& L = c->L;
     FieldMap fm{};
@@ -306,7 +314,11 @@ cudaError_t launch_unpack(Ctx* c, const double* slots, double* const* fields, in
         cudaError_t e = cudaMemsetAsync((void*)slots, 0, sizeof(double) * c->vec_elems(), c->stream);
         if (e != cudaSuccess) return e;
     }
-    k_slots_fields<<<slot_grid(L), dim3(32, 8), 0, c->stream>>>(L, slots, (double*)slots, to_fields, c->nf, 0, fm, 0);
+    const dim3 g = slot_grid(L), blk(32, 8);
+    double* dst = (double*)slots;
+    if (to_fields == 2) k_slots_fields<2><<<g, blk, 0, c->stream>>>(L, c->A, slots, nullptr, c->nf, fm);
+    else if (to_fields) k_slots_fields<1><<<g, blk, 0, c->stream>>>(L, c->A, slots, nullptr, c->nf, fm);
+    else k_slots_fields<0><<<g, blk, 0, c->stream>>>(L, c->A, nullptr, dst, c->nf, fm);
     return cudaGetLastError();
 }
 

@@ -231,7 +231,7 @@ stokes_status stokes_create(stokes_ctx* out, const stokes_grid* g, void* stream)
     if (e == cudaSuccess) e = dalloc(c, (void**)&c.sc, 2 * sizeof(CgScalars));
     if (e == cudaSuccess) e = dalloc(c, (void**)&c.partial, sizeof(double) * 2 * (c.ntiles_all + 32));
     if (e == cudaSuccess) e = dalloc(c, (void**)&c.counter, sizeof(unsigned) * 4);
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&c.h_sc, 2 * sizeof(CgScalars));
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&c.h_sc, 3 * sizeof(CgScalars));
     double** v64[] = {&c.w64.x, &c.w64.r, &c.w64.z, &c.w64.p[0], &c.w64.p[1], &c.w64.q, &c.b64, &c.x64, &c.y64};
     for (double** p : v64)
         if (e == cudaSuccess) e = dalloc(c, (void**)p, sizeof(double) * V);
@@ -256,7 +256,10 @@ stokes_status stokes_destroy(stokes_ctx h) {
     for (auto& ge : c.graph)
         if (ge) cudaGraphExecDestroy(ge);
     for (void* p : c.allocs) cudaFree(p);
-    for (void* p : c.sw_allocs) cudaFree(p);
+    cudaFree(c.sw_grid);
+    cudaFree(c.sw_patch);
+    for (auto& ev : c.sw_ev)
+        if (ev) cudaEventDestroy(ev);
     delete c.sw;
     if (c.h_sc) cudaFreeHost(c.h_sc);
     for (auto& ev : c.ev)

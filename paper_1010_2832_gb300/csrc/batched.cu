@@ -845,11 +845,10 @@ stokes_status stokes_batch_solve(stokes_batch b, const stokes_batch_io* io, stok
     }
     cudaError_t e = cudaSuccess;
     if (b->sw) {
-        // the contexts' Schwarz plans are rebuilt (all their buffers
-        // reallocated) after every weight build: refresh the instance table
-        // and patch list when any plan was rebuilt since the last upload.
-        // (Comparing one buffer's address is not enough: the allocator may
-        // hand that one back at the same address and move the others.)
+        // the contexts' Schwarz plans are rebuilt (other patches, and buffers
+        // that may have moved) after every weight build: refresh the instance
+        // table and patch list when any plan was rebuilt since the last upload.
+        // (Comparing a buffer's address is not enough: it often stays.)
         bool moved = false;
         for (int i = 0; i < b->n; ++i) {
             const SchwarzPlan* P = nullptr;

@@ -97,10 +97,12 @@ struct Ctx {
     int wait_test = 0;          // options.wait_test of the solve in progress (0 outside a solve)
     // additive Schwarz preconditioner (2D), rebuilt lazily after each weight build
     struct SchwarzPlan* sw = nullptr;
-    std::vector<void*> sw_allocs;
+    void* sw_grid = nullptr;     // per patch of the grid: flags, ids, corners, local results
+    void* sw_patch = nullptr;    // per active patch: factors, scalings, maps (room for sw_cap)
+    int sw_cap = 0;
+    cudaEvent_t sw_ev[2]{};      // around the factorisation
     bool sw_ready = false;
-    unsigned sw_epoch = 0;       // incremented by every plan build (its buffers are reallocated)
-    double sw_setup_ms = 0.0;
+    unsigned sw_epoch = 0;       // incremented by every plan build (its buffers may move)
     // transport step (advect.cu): staged velocity and validity, allocated on first use
     void* adv_scratch = nullptr;
 

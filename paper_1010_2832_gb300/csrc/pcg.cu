@@ -225,63 +225,118 @@ __global__ void __launch_bounds__(256, UPD ? 3 : 5) k_sw_finish(Layout L, const 
     });
 }
 
-// Patch plan and local inverses (after every weight build, on first use).
+// Ordered compaction of the patch flags (one block; eight flags per thread and
+// round): the compact id of every patch of the grid (-1: none), the corners of
+// the active ones and their number.
+__global__ void __launch_bounds__(1024) k_schwarz_list(const int* __restrict__ flag, int npx, int ng, int* __restrict__ pid,
+                                                       int* __restrict__ corner, int* __restrict__ count) {
+    __shared__ int warp_tot[32];
+    __shared__ int base_s;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    if (t == 0) base_s = 0;
+    __syncthreads();
+    for (int start = 0; start < ng; start += 8 * 1024) {
+        const int q0 = start + 8 * t;
+        unsigned m = 0;
+        for (int k = 0; k < 8; ++k)
+            if (q0 + k < ng && flag[q0 + k]) m |= 1u << k;
+        int incl = __popc(m);
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) warp_tot[w] = incl;
+        __syncthreads();
+        if (w == 0) {
+            int v = warp_tot[lane];
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += u;
+            }
+            warp_tot[lane] = v;
+        }
+        __syncthreads();
+        int id = base_s + (w ? warp_tot[w - 1] : 0) + incl - __popc(m);
+        for (int k = 0; k < 8 && q0 + k < ng; ++k) {
+            const int q = q0 + k;
+            if (m >> k & 1u) {
+                corner[id] = (q % npx) | ((q / npx) << 16);
+                pid[q] = id++;
+            } else {
+                pid[q] = -1;
+            }
+        }
+        __syncthreads();
+        if (t == 0) base_s += warp_tot[31];
+        __syncthreads();
+    }
+    if (t == 0) *count = base_s;
+}
+
+// Patch plan and local inverses (after every weight build, on first use).  The
+// buffers are the context's and stay: those of the patch grid are allocated
+// once, those of the active patches when there are more of them than before (by
+// an eighth more).  The list is made on the device and the host waits for its
+// length alone, not for the factors.  (Eight allocations and frees, the list on
+// the host and a wait for the factors took 0.30 ms of a 150^2 jet step.)
 static cudaError_t schwarz_build(Ctx* c) {
     const Layout& L = c->L;
+    cudaStream_t s = c->stream;
     cudaError_t e;
-    for (void* p : c->sw_allocs) cudaFree(p);
-    c->sw_allocs.clear();
     ++c->sw_epoch;
+    c->sw_ready = false;
     if (!c->sw) c->sw = new SchwarzPlan();
     SchwarzPlan& P = *c->sw;
-    P.npx = (L.nx + 1 + PB - 1) / PB;
-    P.npy = (L.ny + 1 + PB - 1) / PB;
-    const int ng = P.npx * P.npy;
-    auto al = [&](void** p, size_t bytes) -> cudaError_t {
-        cudaError_t r = cudaMalloc(p, bytes ? bytes : 16);
-        if (r == cudaSuccess) c->sw_allocs.push_back(*p);
-        return r;
-    };
-    int* dflag = nullptr;
-    if ((e = al((void**)&dflag, sizeof(int) * ng)) != cudaSuccess) return e;
-    k_schwarz_mark<<<dim3((P.npx + 127) / 128, P.npy), 128, 0, c->stream>>>(L, c->A, P.npx, P.npy, dflag);
-    std::vector<int> flag(ng), pid(ng, -1), corner;
-    if ((e = cudaMemcpyAsync(flag.data(), dflag, sizeof(int) * ng, cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess)
-        return e;
-    if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return e;
-    for (int J = 0; J < P.npy; ++J)
-        for (int I = 0; I < P.npx; ++I)
-            if (flag[J * P.npx + I]) { pid[J * P.npx + I] = (int)corner.size(); corner.push_back(I | (J << 16)); }
-    P.np = (int)corner.size();
+    const int npx = (L.nx + 1 + PB - 1) / PB, npy = (L.ny + 1 + PB - 1) / PB, ng = npx * npy;
+    if (!c->sw_grid) {
+        // flags, ids, corners and the count (ints), then the local results
+        const size_t ints = ((size_t)3 * ng + 4 + 63) / 64 * 64 * sizeof(int);
+        if ((e = cudaMalloc(&c->sw_grid, ints + sizeof(float) * (size_t)ng * PMAX)) != cudaSuccess) { c->sw_grid = nullptr; return e; }
+        P.npx = npx;
+        P.npy = npy;
+        P.pid = (int*)c->sw_grid + ng;
+        P.corner = (int*)c->sw_grid + 2 * (size_t)ng;
+        P.ybuf = (float*)((char*)c->sw_grid + ints);
+        for (cudaEvent_t& ev : c->sw_ev)
+            if (!ev && (e = cudaEventCreate(&ev)) != cudaSuccess) return e;
+    }
+    int* const flag = (int*)c->sw_grid;
+    int* const count = (int*)c->sw_grid + 3 * (size_t)ng;
+    int* const h_count = (int*)(c->h_sc + 2);
+    k_schwarz_mark<<<dim3((npx + 127) / 128, npy), 128, 0, s>>>(L, c->A, npx, npy, flag);
+    k_schwarz_list<<<1, 1024, 0, s>>>(flag, npx, ng, P.pid, P.corner, count);
+    if ((e = cudaMemcpyAsync(h_count, count, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(P.ybuf, 0, sizeof(float) * (size_t)ng * PMAX, s)) != cudaSuccess) return e;
+    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+    P.np = *h_count;
     P.evict_first = sw_factors_exceed_l2((size_t)P.np * SW_FAC_BYTES) ? 1 : 0;
-    const size_t np = std::max(1, P.np);
-    if ((e = al((void**)&P.pid, sizeof(int) * ng)) != cudaSuccess) return e;
-    if ((e = al((void**)&P.corner, sizeof(int) * np)) != cudaSuccess) return e;
-    if ((e = al((void**)&P.nloc, sizeof(int) * np)) != cudaSuccess) return e;
-    if ((e = al((void**)&P.lmap, sizeof(short) * np * PMAX)) != cudaSuccess) return e;
-    // FP16 factors with a FP32 scale per row (BF16 storage needed 4.4x the CG
-    // iterations on the 1024^2 bump workload; FP16 about 1.02x)
-    if ((e = al((void**)&P.fac, (size_t)SW_FAC_BYTES * np)) != cudaSuccess) return e;
-    if ((e = al((void**)&P.scale, sizeof(float) * np * PMAX)) != cudaSuccess) return e;
-    if ((e = al((void**)&P.ybuf, sizeof(float) * ng * PMAX)) != cudaSuccess) return e;
-    cudaMemcpyAsync(P.pid, pid.data(), sizeof(int) * ng, cudaMemcpyHostToDevice, c->stream);
-    if (P.np) cudaMemcpyAsync(P.corner, corner.data(), sizeof(int) * P.np, cudaMemcpyHostToDevice, c->stream);
-    cudaMemsetAsync(P.ybuf, 0, sizeof(float) * ng * PMAX, c->stream);
+    if (!c->sw_patch || P.np > c->sw_cap) {
+        if (c->sw_patch) cudaFree(c->sw_patch);
+        c->sw_patch = nullptr;
+        c->sw_cap = 0;
+        const size_t cap = std::min((size_t)ng, (size_t)P.np + P.np / 8 + 8);
+        // FP16 factors with a FP32 scale per row (BF16 storage needed 4.4x the CG
+        // iterations on the 1024^2 bump workload; FP16 about 1.02x), scalings,
+        // local maps, sizes
+        auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+        const size_t f = up((size_t)SW_FAC_BYTES * cap), sc = up(sizeof(float) * cap * PMAX), lm = up(sizeof(short) * cap * PMAX);
+        if ((e = cudaMalloc(&c->sw_patch, f + sc + lm + sizeof(int) * cap)) != cudaSuccess) { c->sw_patch = nullptr; return e; }
+        c->sw_cap = (int)cap;
+        char* base = (char*)c->sw_patch;
+        P.fac = (uint8_t*)base;
+        P.scale = (float*)(base + f);
+        P.lmap = (short*)(base + f + sc);
+        P.nloc = (int*)(base + f + sc + lm);
+    }
     const int smem = SW_SETUP_SMEM;
     cudaFuncSetAttribute(k_schwarz_setup, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     cudaFuncSetAttribute(k_schwarz_gemv, cudaFuncAttributeMaxDynamicSharedMemorySize, SW_GEMV_SMEM);
-    cudaEvent_t a, b;
-    cudaEventCreate(&a); cudaEventCreate(&b);
-    cudaEventRecord(a, c->stream);
-    if (P.np) k_schwarz_setup<<<P.np, 256, smem, c->stream>>>(L, c->A, c->A.coef64, P);
-    cudaEventRecord(b, c->stream);
-    if ((e = cudaEventSynchronize(b)) != cudaSuccess) return e;
-    float ms = 0;
-    cudaEventElapsedTime(&ms, a, b);
-    cudaEventDestroy(a); cudaEventDestroy(b);
-    c->sw_setup_ms = ms;
+    cudaEventRecord(c->sw_ev[0], s);
+    if (P.np) k_schwarz_setup<<<P.np, 256, smem, s>>>(L, c->A, c->A.coef64, P);
+    cudaEventRecord(c->sw_ev[1], s);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     c->sw_ready = true;
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 // CTAs of a persistent tile kernel: min(tiles, the CTAs resident on the
@@ -716,12 +771,21 @@ cudaError_t apply_preconditioner(Ctx* c, int which, const float* r, float* z) {
     return c->h_sc[0].status == STOKES_ERR_TIMEOUT ? cudaErrorLaunchTimeout : cudaSuccess;
 }
 
-double schwarz_setup_ms(Ctx* c) { return c->sw_ready ? c->sw_setup_ms : -1.0; }
+// device time of the last plan's factorisation (waits for it)
+double schwarz_setup_ms(Ctx* c) {
+    float ms = -1.f;
+    if (!c->sw_ready || cudaEventSynchronize(c->sw_ev[1]) != cudaSuccess ||
+        cudaEventElapsedTime(&ms, c->sw_ev[0], c->sw_ev[1]) != cudaSuccess)
+        return -1.0;
+    return ms;
+}
 
 // The context's Schwarz plan for its current weights, built if needed.
 cudaError_t schwarz_ensure(Ctx* c, const SchwarzPlan** plan) {
     cudaError_t e = cudaSuccess;
     if (!c->sw_ready) e = schwarz_build(c);
+    // (the caller, the batched solver, reads the plan on a stream of its own)
+    if (e == cudaSuccess) e = cudaEventSynchronize(c->sw_ev[1]);
     if (plan) *plan = c->sw;
     return e;
 }

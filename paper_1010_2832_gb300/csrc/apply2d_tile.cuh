@@ -27,15 +27,16 @@ template <class T, int TY> struct Smem2 {
 
 // Apply on the tile whose lower corner is (c0, r0) in padded coordinates.
 // x: input (CG mode: z, with p = z + beta pold written to pnew); y: output;
-// b: RESID right-hand side.  Returns the warp sum of this warp's partial dot
-// (x.y in CG mode, y.y in RESID mode); the caller combines warps.
-template <class T, class C, int MODE, int TY, int NT>
-__device__ double apply2d_tile(const Layout& L, int c0, int r0, const Coef<C>& cf, const T* __restrict__ x,
+// b: RESID right-hand side.  Returns this thread's partial dot (FP64; x.y in CG
+// mode, y.y in RESID mode; nothing past the first TY warps); the caller combines.
+// grp: the NT threads that take the tile (a CTA, or part of one with its barrier).
+template <class T, class C, int MODE, int TY, int NT, class G>
+__device__ double apply2d_tile(const G& grp, const Layout& L, int c0, int r0, const Coef<C>& cf, const T* __restrict__ x,
                                T* __restrict__ y, const T* __restrict__ pold, T* __restrict__ pnew, T beta,
                                const T* __restrict__ b, Smem2<T, TY>& sm) {
     const int64_t S = L.stride;
     const C *a_c = cf.f[0], *a_n = cf.f[1], *d_c = cf.f[2], *d_n = cf.f[3], *K_u = cf.f[4], *K_v = cf.f[5];
-    const int t = threadIdx.x;
+    const int t = grp.thread();
     // Every global load of the tile is issued up front (face coefficients and
     // the own slots' coefficients into registers), so one CTA waits for one
     // memory round trip rather than three.
@@ -78,7 +79,7 @@ __device__ double apply2d_tile(const Layout& L, int c0, int r0, const Coef<C>& c
         sm.V[jj][ii] = ac * (p + txx);
         sm.N[jj][ii] = an * txy;
     }
-    __syncthreads();
+    grp.sync();
 #pragma unroll
     for (int q = 0; q < NFACE; ++q) {
         int e = t + q * NT;
@@ -88,7 +89,7 @@ __device__ double apply2d_tile(const Layout& L, int c0, int r0, const Coef<C>& c
             sm.Zv[jj][ii] = kv[q] * ((sm.V[jj + 1][ii] - sm.V[jj][ii]) + (sm.N[jj + 1][ii] - sm.N[jj + 1][ii + 1]));
         }
     }
-    __syncthreads();
+    grp.sync();
     Acc<T> acc;
 #pragma unroll
     for (int q = 0; q < NOWN; ++q) {
@@ -103,12 +104,12 @@ __device__ double apply2d_tile(const Layout& L, int c0, int r0, const Coef<C>& c
         T yp, yxx;
         if (ac != T(0)) {
             yp = ac * ((zu - zur) + (zv - zvu));
-            yxx = dc * txx + ac * ((zur - zu) + (zv - zvu));
+            yxx = fma(dc, txx, ac * ((zur - zu) + (zv - zvu)));
         } else {
             yp = p_;
             yxx = txx;
         }
-        T yxy = dn * txy + an * ((zu - zud) + (zv - zvl));
+        T yxy = fma(dn, txy, an * ((zu - zud) + (zv - zvl)));
         if (MODE == MODE_RESID) {
             yxx = b[o] - yxx; yxy = b[S + o] - yxy; yp = b[2 * S + o] - yp;
         }
@@ -116,7 +117,8 @@ __device__ double apply2d_tile(const Layout& L, int c0, int r0, const Coef<C>& c
         if (MODE == MODE_RESID) { acc.add(yxx, yxx); acc.add(yxy, yxy); acc.add(yp, yp); }
         else if (MODE == MODE_CG) { acc.add(txx, yxx); acc.add(txy, yxy); acc.add(p_, yp); }
     }
-    return MODE == MODE_PLAIN ? 0.0 : acc.warp();
+    static_assert(sizeof(T) == 8, "the partial dot is a double");
+    return MODE == MODE_PLAIN ? 0.0 : acc.s;
 }
 
 }  // namespace stk

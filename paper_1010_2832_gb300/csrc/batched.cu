@@ -10,13 +10,23 @@
 //   C  (Schwarz only) local patch solves on r - alpha q (r in CHECK mode)
 //   D  CG instances: x += alpha p, r -= alpha q; every instance:
 //      z = M^-1 r (Jacobi, or the gather of the local results), r.z, r.r
-// The CTA that reports an instance's last tile of a phase reduces that
-// instance's per-tile partials in list order (deterministic) and updates
+// The CTA (or half CTA) that reports an instance's last tile of a phase reduces
+// that instance's per-tile partials in list order (deterministic) and updates
 // its scalars: CG -> CHECK when the recurrence residual meets the
 // tolerance; CHECK -> done if the true residual meets it, else CG restarts
 // from the true residual.  Instances retire independently; the kernel ends
 // when all have.  Every grid barrier is a bounded wait: after ~2^24 polls
 // it records STOKES_ERR_TIMEOUT and every CTA returns.
+//
+// What bounds it: latency.  A pass over 12 instances of 64..160 cells a side (776
+// tiles of 32 x 4, 3,937 patches, 3 CTAs per SM) moves 20 MB that L2 holds and does
+// little arithmetic, and takes 79 k cycles (41 us): A 28 k of which up to 20 k are the
+// FP64 pipe of the fullest SM (about 195 warp instructions a tile at 64 clocks of a
+// quarter SM), C 32 k (26 patches an SM, six at a time), D 20 k; 9 k of A and D
+// each are the sums, an instance's totals and the barrier.  It was 134 k cycles
+// (70 us) with one patch and one 4-row tile per CTA at a time (half its warps
+// idle), a fence at each step of a sum, scalars read one by one, a barrier that
+// counted and then released, and the gathers of the three fields one after another.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -30,6 +40,7 @@
 #include "internal.cuh"
 #include "ctx.cuh"
 #include "apply2d_tile.cuh"
+#include "reduce.cuh"
 #include "schwarz_plan.cuh"
 
 namespace stk {
@@ -57,136 +68,196 @@ struct BInst {
     const uint8_t* act_node;
 };
 
-struct BState {
+struct alignas(16) BState {
     double rz, rr, alpha, beta, tol2, bb;
     int mode;      // 0 CG, 1 CHECK (true residual), 2 START (Schwarz: first z = M^-1 b pending)
     int parity, iter, done, status;
     unsigned cnt;
 };
 
-struct BGlobal {
-    unsigned bar_count, bar_gen;
-    int ndone, err;
+// One 16-byte word, so a poll of the grid barrier reads all of it at once.
+struct alignas(16) BGlobal {
+    unsigned bar_count;          // arrivals since the launch began
+    int ndone;                   // instances done; changes in the initial phase and phase D only
+    int err, pad;
 };
 
-__device__ bool grid_sync(BGlobal* g, unsigned nblocks) {
-    __shared__ int ok;
+// Grid barrier: the CTAs' arrivals are counted up through the launch and each CTA
+// polls for this barrier's total, so no CTA has to see the last arrival and
+// release the others (one L2 round trip and one fence less than a count and a
+// generation).  Bounded; false, for the whole CTA, after an error anywhere.
+// ndone: the instances done as of this barrier (meaningful after phase D).
+__device__ __forceinline__ bool grid_sync(BGlobal* g, unsigned nblocks, unsigned& target, int* ndone = nullptr) {
+    __shared__ int ok, nd;
+    target += nblocks;
     __syncthreads();
     if (threadIdx.x == 0) {
-        ok = 1;
-        volatile unsigned* genp = &g->bar_gen;
-        volatile int* errp = &g->err;
-        unsigned gen = *genp;
-        __threadfence();
-        unsigned arrived = atomicAdd(&g->bar_count, 1u) + 1u;
-        if (arrived == nblocks) {
-            g->bar_count = 0u;
-            __threadfence();
-            atomicAdd(&g->bar_gen, 1u);
-        } else {
-            long long spins = 0;
-            while (*genp == gen) {
-                if (*errp) { ok = 0; break; }
-                if (++spins > (1LL << 24)) { atomicExch(&g->err, (int)STOKES_ERR_TIMEOUT); ok = 0; break; }
-                __nanosleep(64);
-            }
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&g->bar_count) : "memory");
+        unsigned count;
+        int done, err, pad;
+        for (int spins = 0;; ++spins) {
+            asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(count), "=r"(done), "=r"(err), "=r"(pad)
+                         : "l"(g)
+                         : "memory");
+            if (err || (int)(count - target) >= 0) break;
+            if (spins > (1 << 24)) { err = (int)STOKES_ERR_TIMEOUT; atomicExch(&g->err, err); }
         }
-        __threadfence();
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        ok = err == 0;
+        nd = done;
     }
     __syncthreads();
-    return ok && !((volatile int*)&g->err)[0];
+    if (ndone) *ndone = nd;
+    return ok;
 }
 
-// Block-reduce two warp partials, store them for tile w, and let the CTA that
-// completes instance i's phase reduce all of i's tiles; fin(s0, s1) runs on
-// thread 0 of that CTA.
-template <class Fin>
-__device__ void tile_report(double v0, double v1, double* part, int w, BState* st, const BInst& I, Fin fin) {
-    __shared__ double red[2][8];
-    __shared__ bool last;
-    int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    if (lane == 0) { red[0][wp] = v0; red[1][wp] = v1; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s0 = 0.0, s1 = 0.0;
-        for (int q = 0; q < 8; ++q) { s0 += red[0][q]; s1 += red[1][q]; }
-        part[2 * w] = s0;
-        part[2 * w + 1] = s1;
-        __threadfence();
-        unsigned prev = atomicAdd(&st->cnt, 1u);
-        last = (prev == (unsigned)(I.te - I.tb) - 1u);
+// The CTA's threads take a tile of 16 or 8 rows together and tiles of 4 rows by
+// halves, two tiles at a time (4 rows occupy 4 warps).
+template <int TY> struct TileGroups {
+    static constexpr int NG = TY == 4 ? 2 : 1, NT = 256 / NG, NW = NT / 32;
+    using Group = typename std::conditional<NG == 2, BarGroup, CtaGroup>::type;
+    static __device__ Group make() {
+        if constexpr (NG == 2) return BarGroup{(int)threadIdx.x & 127, 1 + ((int)threadIdx.x >> 7)};
+        else return CtaGroup{};
     }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    double s0 = 0.0, s1 = 0.0;
-    for (int k = I.tb + threadIdx.x; k < I.te; k += 256) {
-        s0 += ((volatile double*)part)[2 * k];
-        s1 += ((volatile double*)part)[2 * k + 1];
+};
+struct ReportSmem {
+    double red[16];
+    BState st;
+    bool last;
+};
+
+// Sum a tile's accumulators (Q per thread of the group; its first TY warps hold
+// them), store them for tile w, and let the group that completes instance i's
+// phase reduce all of i's tiles; fin(sums, state) runs on one thread of that group
+// on a copy of the state, which is read while the tiles' sums are and written back
+// whole (field by field its reads queue behind its writes, an L2 latency each).  FP64
+// instructions are slow on this part (see reduce.cuh): warps without rows take no
+// part, two sums share a tree and a chain.  The order of the additions: a warp's
+// xor tree, the warps one after another; then (virtual) thread t of 256 adds the
+// tiles t, t + 256, ..., and the trees and the warps again.
+template <int TY, int Q, class G, class Fin>
+__device__ void tile_report(const G& grp, ReportSmem& sm, const double (&acc)[Q], double* part, int w, BState* st,
+                            const BInst& I, Fin fin) {
+    constexpr int NW = TileGroups<TY>::NW, ROWS = TY < NW ? TY : NW;
+    const int t = grp.thread(), lane = t & 31, wp = t >> 5;
+    if (wp < ROWS) {
+        const double s = warp_sums(acc);
+        if (lane == 0) sm.red[wp * Q] = s;
+        if (Q == 2 && lane == 16) sm.red[wp * Q + 1] = s;
     }
-    s0 = warp_sum(s0);
-    s1 = warp_sum(s1);
-    __syncthreads();
-    if (lane == 0) { red[0][wp] = s0; red[1][wp] = s1; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t0 = 0.0, t1 = 0.0;
-        for (int q = 0; q < 8; ++q) { t0 += red[0][q]; t1 += red[1][q]; }
-        fin(t0, t1);
-        st->cnt = 0u;
-        __threadfence();
+    grp.sync();
+    const int n = I.te - I.tb;
+    if (wp == 0) {
+        if (lane < Q) {
+            double s = sm.red[lane];
+#pragma unroll
+            for (int q = 1; q < ROWS; ++q) s += sm.red[q * Q + lane];
+            part[2 * w + lane] = s;
+        }
+        __syncwarp();
+        if (lane == 0) {
+            unsigned before;
+            asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(before) : "l"(&st->cnt) : "memory");
+            sm.last = before == (unsigned)n - 1u;
+        }
     }
-    __syncthreads();
+    grp.sync();
+    if (!sm.last) return;
+    static_assert(sizeof(BState) % 16 == 0 && sizeof(BState) <= 512, "one 16-byte word per lane");
+    uint4* const copy = reinterpret_cast<uint4*>(&sm.st);
+    const bool mover = t < (int)sizeof(BState) / 16;
+    if (mover) copy[t] = __ldcg(reinterpret_cast<const uint4*>(st) + t);
+    const int nw = min((n + 31) / 32, 8);
+    for (int vw = wp; vw < nw; vw += NW) {
+        double v[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) v[q] = 0.0;
+        for (int k = I.tb + 32 * vw + lane; k < I.te; k += 256)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) v[q] += ((volatile double*)part)[2 * k + q];
+        __syncwarp();
+        const double s = warp_sums(v);
+        if (lane == 0) sm.red[vw * Q] = s;
+        if (Q == 2 && lane == 16) sm.red[vw * Q + 1] = s;
+    }
+    grp.sync();
+    if (wp == 0) {
+        double s = 0.0;
+        if (lane < Q) {
+            s = sm.red[lane];
+            for (int q = 1; q < nw; ++q) s += sm.red[q * Q + lane];
+        }
+        double tot[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) tot[q] = __shfl_sync(0xffffffffu, s, q);
+        if (lane == 0) {
+            fin(tot, &sm.st);
+            sm.st.cnt = 0u;
+        }
+        __syncwarp();
+        if (mover) reinterpret_cast<uint4*>(st)[t] = copy[t];
+    }
+    grp.sync();
 }
 
-// Additive Schwarz local solve of patch p of instance I, by the whole CTA
-// (256 threads; the triangular products use 128): the same arithmetic as
-// the single-system kernel k_schwarz_gemv, on r_eff = r - alpha q read in
-// FP64 (alpha = 0 outside a CG step).  Thread 0 starts the bulk copy of the
-// factor and waits on the CTA's mbarrier (phase parity = uses & 1, bounded);
-// a copy that never completes sets the batch's error flag.
-__device__ void batched_local_solve(const BInst& I, int p, double alpha, uint8_t* Fs, float* s, float* y, __half* hb,
-                                    unsigned long long* bar, uint32_t& uses, int& ok_s, BGlobal* g) {
+// Additive Schwarz local solve of patch p of instance I, by 128 threads of the
+// CTA (it solves two patches at a time; with one, half of its warps idled through
+// the products): the same arithmetic as the single-system kernel k_schwarz_gemv,
+// on r_eff = r - alpha q read in FP64 (alpha = 0 outside a CG step).  The bulk copy
+// of the factor is in flight on entry; thread 0 of the group waits for it on the
+// group's mbarrier (phase parity = uses & 1, bounded).  The next patch's copy starts
+// as soon as this one's products are done.  A copy that never completes sets the
+// batch's error flag, and the group (false) starts no further one.
+struct PatchRef {
+    int inst, p, n, corner;
+    bool on;                        // the instance is not done
+};
+__device__ __forceinline__ void patch_issue(const BInst& I, const PatchRef& c, uint8_t* Fs, unsigned long long* bar) {
+    sw_issue(smem_u32(bar), Fs, I.sw.fac + (int64_t)c.p * SW_FAC_BYTES, sw_patch_bytes(c.n), I.sw.evict_first != 0);
+}
+__device__ __forceinline__ bool batched_local_solve(const BarGroup& grp, const BInst* inst, const BState* st,
+                                                    const PatchRef& cur, const PatchRef& next, uint8_t* Fs, float* s,
+                                                    float* raw, __half* hb, unsigned long long* bar, uint32_t& uses,
+                                                    int& ok_s, BGlobal* g) {
+    const BInst& I = inst[cur.inst];
     const SchwarzPlan& P = I.sw;
     const Layout& L = I.L;
-    const int t = threadIdx.x;
-    // after an error (a copy that timed out) start no further copies; the
-    // decision is the same for the whole CTA
-    if (t == 0) ok_s = ((volatile int*)&g->err)[0] == 0;
-    __syncthreads();
-    if (!ok_s) return;
-    const int n = P.nloc[p];
+    const int t = grp.t, p = cur.p, n = cur.n;
     const uint32_t b_addr = smem_u32(bar);
-    if (t == 0) sw_issue(b_addr, Fs, P.fac + (int64_t)p * SW_FAC_BYTES, sw_patch_bytes(n), P.evict_first != 0);
+    const volatile BState* vs = st + cur.inst;
+    const int mode = vs->mode;
+    const double step = vs->alpha, alpha = mode == 0 ? step : 0.0;
     constexpr float H = 0.70710678118654752f;
-    const int CI = P.corner[p] & 0xffff, CJ = P.corner[p] >> 16;
+    const int CI = cur.corner & 0xffff, CJ = cur.corner >> 16;
     const int a0 = PB * CI - 1, b0 = PB * CJ - 1;
     const short* map = P.lmap + (int64_t)p * PMAX;
     const float* scl = P.scale + (int64_t)p * PMAX;
-    int kk = -1, kp = -1;
-    float sa = 0.f, sb = 0.f;
-    if (t < 2 * PR * PR) {
-        const int e = t;
-        const int rem = e % (PR * PR), jj = rem / PR, ii = rem % PR;
-        const int64_t o = L.off(a0 + ii + 1, b0 + jj + 1, 0);
+    // One entry per thread (FP64 instructions are slow: see reduce.cuh), fields 0
+    // and 2 of a sample exchange theirs; e2 is the partner's entry (field 1: none).
+    const int e = t, f = e / (PR * PR), e2 = f == 1 ? e : f == 0 ? e + 2 * PR * PR : e - 2 * PR * PR;
+    int kk = -1, k2 = -1;
+    float sa = 0.f, sb = 0.f, v = 0.f;
+    if (e < PMAX) {
+        const int rem = e - f * PR * PR, jj = rem / PR, ii = rem % PR;
+        const int64_t o = f * L.stride + L.off(a0 + ii + 1, b0 + jj + 1, 0);
         kk = map[e];
         sa = scl[e];
-        if (e >= PR * PR) {
-            const float rv = (float)(I.r[L.stride + o] - alpha * I.q[L.stride + o]);
-            if (kk >= 0) s[kk] = rv * sa;
+        if (f != 1) {
+            k2 = map[e2];
+            sb = scl[e2];
+        }
+        v = (float)(I.r[o] - alpha * I.q[o]);
+        raw[e] = v;
+    }
+    grp.sync();
+    if (kk >= 0) {
+        if (k2 >= 0) {
+            const float w = raw[e2];
+            s[kk] = (f == 0 ? v + w : w - v) * H * sa;
         } else {
-            kp = map[2 * PR * PR + e];
-            sb = scl[2 * PR * PR + e];
-            const float rt = (float)(I.r[o] - alpha * I.q[o]);
-            const float rp = (float)(I.r[2 * L.stride + o] - alpha * I.q[2 * L.stride + o]);
-            if (kk >= 0 && kp >= 0) {
-                s[kk] = (rt + rp) * H * sa;
-                s[kp] = (rt - rp) * H * sb;
-            } else if (kk >= 0) {
-                s[kk] = rt * sa;
-            } else if (kp >= 0) {
-                s[kp] = rp * sb;
-            }
+            s[kk] = v * sa;
         }
     }
     if (t >= n && t < (n + 7) / 8 * 8) s[t] = 0.f;
@@ -194,64 +265,64 @@ __device__ void batched_local_solve(const BInst& I, int p, double alpha, uint8_t
         ok_s = mbar_wait(b_addr, uses & 1u) ? 1 : 0;
         ++uses;
     }
-    __syncthreads();
+    grp.sync();
     if (!ok_s) {
         if (t == 0) {
             mbar_wait(b_addr, (uses - 1u) & 1u);
             atomicExch(&g->err, (int)STOKES_ERR_TIMEOUT);
         }
-        __syncthreads();
-        return;
+        return false;
     }
-    sw_factor_products(Fs, n, s, y, hb);
+    sw_factor_products(grp, Fs, n, s, s, hb);
+    if (t == 0 && next.on) patch_issue(inst[next.inst], next, Fs, bar);
     float* out = P.ybuf + (int64_t)(CJ * P.npx + CI) * PMAX;
-    if (t < 2 * PR * PR) {
-        const int e = t;
-        if (e >= PR * PR) {
-            if (kk >= 0) out[e] = s[kk] * sa;
-        } else if (kk >= 0 && kp >= 0) {
-            const float a = s[kk] * sa, b = s[kp] * sb;
-            out[e] = (a + b) * H;
-            out[2 * PR * PR + e] = (a - b) * H;
-        } else if (kk >= 0) {
-            out[e] = s[kk] * sa;
-        } else if (kp >= 0) {
-            out[2 * PR * PR + e] = s[kp] * sb;
-        }
+    if (kk >= 0 && k2 >= 0) {
+        // field 0's product is the fused one in both
+        out[e] = (f == 0 ? fmaf(s[kk], sa, __fmul_rn(s[k2], sb)) : fmaf(s[k2], sb, -__fmul_rn(s[kk], sa))) * H;
+    } else if (kk >= 0) {
+        out[e] = s[kk] * sa;
     }
-    __syncthreads();                             // the next patch reuses shared memory
+    grp.sync();                                  // the next patch reuses shared memory
+    return true;
 }
 
-// z of field f at sample (i, j) from the patches' local results (the
-// single-system gather schwarz_gather_slot, in FP64 out).
-__device__ __forceinline__ double batched_gather(const BInst& I, int f, int i, int j, double r) {
+// z of the three fields at sample (i, j) from the patches' local results (the
+// single-system gather schwarz_gather_slot, in FP64 out).  The fields share the
+// window and their loads go out together; an entry that is not the patch's own
+// (an inactive unknown) is read and not used.
+__device__ __forceinline__ void batched_gather(const BInst& I, int i, int j, const double (&r)[3], double (&z)[3]) {
     const Layout& L = I.L;
-    if (!unknown_active(I.act_cell, I.act_node, L, f, i, j))
-        return (i >= 0 && j >= 0 && i <= L.nx && j <= L.ny) ? r : 0.0;
     const SchwarzPlan& P = I.sw;
     const int ilo = max((i + PB - 1) / PB - 1, 0), ihi = min((i + 1) / PB, P.npx - 1);
     const int jlo = max((j + PB - 1) / PB - 1, 0), jhi = min((j + 1) / PB, P.npy - 1);
     // (a loop over the patches in range: a fixed, masked 2 x 2 window as in
     // the single-system gather needs more registers here, which costs this
     // persistent kernel a CTA per SM)
-    float s = 0.f;
+    float s[3] = {0.f, 0.f, 0.f};
     for (int J = jlo; J <= jhi; ++J)
         for (int Ip = ilo; Ip <= ihi; ++Ip) {
             const int ii = i - (PB * Ip - 1), jj = j - (PB * J - 1);
-            s += P.ybuf[(int64_t)(J * P.npx + Ip) * PMAX + (f * PR + jj) * PR + ii];
+            const float* y = P.ybuf + (int64_t)(J * P.npx + Ip) * PMAX + jj * PR + ii;
+#pragma unroll
+            for (int f = 0; f < 3; ++f) s[f] += y[f * PR * PR];
         }
-    return (double)s;
+    const bool in = i >= 0 && j >= 0 && i <= L.nx && j <= L.ny;
+#pragma unroll
+    for (int f = 0; f < 3; ++f)
+        z[f] = unknown_active(I.act_cell, I.act_node, L, f, i, j) ? (double)s[f] : in ? r[f] : 0.0;
 }
 
 template <int TY, bool SW>
 struct BatchedSmem {
-    static constexpr int APPLY = (int)sizeof(Smem2<double, TY>);
-    static constexpr int LOCAL = SW ? SW_FAC_BYTES : 0;
+    static constexpr int TILE = (int)(sizeof(Smem2<double, TY>) + 127) / 128 * 128;
+    static constexpr int APPLY = TileGroups<TY>::NG * TILE;
+    static constexpr int FAC = (SW_FAC_BYTES + 127) / 128 * 128;
+    static constexpr int LOCAL = SW ? 2 * FAC : 0;
     static constexpr int BYTES = APPLY > LOCAL ? APPLY : LOCAL;
 };
 
 template <int TY, bool SW>
-__global__ void __launch_bounds__(256) k_batched(const BInst* __restrict__ inst, BState* st,
+__global__ void __launch_bounds__(256, TY == 4 ? 3 : 2) k_batched(const BInst* __restrict__ inst, BState* st,
                                                  const int* __restrict__ wl_inst, const int* __restrict__ wl_c0,
                                                  const int* __restrict__ wl_r0, int nwork,
                                                  const int* __restrict__ pl_inst, const int* __restrict__ pl_patch,
@@ -260,27 +331,39 @@ __global__ void __launch_bounds__(256) k_batched(const BInst* __restrict__ inst,
     // shared memory: the apply's staging (phase A) and the local solves'
     // factor (phase C) never live at the same time
     __shared__ __align__(128) unsigned char smraw[BatchedSmem<TY, SW>::BYTES];
-    Smem2<double, TY>& sm = *reinterpret_cast<Smem2<double, TY>*>(smraw);
-    uint8_t* Fs = reinterpret_cast<uint8_t*>(smraw);
-    __shared__ __align__(16) float ls[SW ? PMAX8 : 4];
-    __shared__ __align__(16) __half lhb[SW ? SW_HB_HALVES : 8];
-    __shared__ __align__(8) unsigned long long lbar;
-    __shared__ int lok;
+    using TG = TileGroups<TY>;
+    constexpr int NG = TG::NG;
+    const typename TG::Group tg = TG::make();     // takes tiles blockIdx.x + nb ti, + NG nb, ...
+    const int ti = threadIdx.x / TG::NT;
+    Smem2<double, TY>& sm = *reinterpret_cast<Smem2<double, TY>*>(smraw + ti * BatchedSmem<TY, SW>::TILE);
+    __shared__ ReportSmem rep_s[NG];
+    ReportSmem& rs = rep_s[ti];
+    const BarGroup grp{(int)threadIdx.x & 127, 1 + ((int)threadIdx.x >> 7)};     // takes patches
+    const int gi = threadIdx.x >> 7;
+    uint8_t* Fs = reinterpret_cast<uint8_t*>(smraw) + gi * (SW ? BatchedSmem<TY, SW>::FAC : 0);
+    __shared__ __align__(16) float ls[2][SW ? (PMAX8 + 3) / 4 * 4 : 4], lraw[2][SW ? PMAX : 4];
+    __shared__ __align__(16) __half lhb[2][SW ? (SW_HB_HALVES + 7) / 8 * 8 : 8];
+    __shared__ __align__(8) unsigned long long lbar[2];
+    __shared__ int lok[2];
     uint32_t uses = 0;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    bool copies = true;
+    unsigned bars = 0;
+    int ndone = 0;
+    const int lane = threadIdx.x & 31, warp = tg.thread() >> 5;
     const unsigned nb = gridDim.x;
-    if (SW && threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&lbar)), "r"(1) : "memory");
+    if (SW && grp.t == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&lbar[gi])), "r"(1) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // ---- init: r = b, x = 0, p = 0; Jacobi: z = M^-1 r (Schwarz: later) --
-    for (int w = blockIdx.x; w < nwork; w += nb) {
+    for (int w = blockIdx.x + nb * ti; w < nwork; w += NG * nb) {
         const int i = wl_inst[w];
         const BInst& I = inst[i];
         const bool swi = SW && I.use_sw;
         const int64_t S = I.L.stride;
-        double rz = 0.0, rr = 0.0;
-        for (int row = warp; row < TY; row += 8) {
+        double sums[2] = {0.0, 0.0};
+        double &rz = sums[0], &rr = sums[1];
+        for (int row = warp; row < TY; row += TG::NW) {
             int64_t o = I.L.off(wl_c0[w] + lane, wl_r0[w] + row, 0);
             for (int f = 0; f < 3; ++f) {
                 int64_t of = f * S + o;
@@ -289,8 +372,8 @@ __global__ void __launch_bounds__(256) k_batched(const BInst* __restrict__ inst,
                 rz = fma(r, z, rz); rr = fma(r, r, rr);
             }
         }
-        BState* s = st + i;
-        tile_report(warp_sum(rz), warp_sum(rr), part, w, s, I, [&](double trz, double trr) {
+        tile_report<TY, 2>(tg, rs, sums, part, w, st + i, I, [&](const double (&tot)[2], BState* s) {
+            const double trz = tot[0], trr = tot[1];
             s->rz = trz; s->rr = trr; s->bb = trr; s->tol2 = tol * tol * trr;
             s->mode = swi ? 2 : 0; s->parity = 0; s->iter = 0; s->beta = 0.0; s->status = 0; s->alpha = 0.0;
             s->done = trr == 0.0 ? 1 : 0;
@@ -298,81 +381,120 @@ __global__ void __launch_bounds__(256) k_batched(const BInst* __restrict__ inst,
             if (s->done) atomicAdd(&g->ndone, 1);
         });
     }
-    if (!grid_sync(g, nb)) return;
+    if (!grid_sync(g, nb, bars, &ndone)) return;
     for (;;) {
-        if (((volatile int*)&g->ndone)[0] >= ninst) return;
+        if (ndone >= ninst) return;
         // ---- phase A: CG: p = z + beta p_old, q = A p, p.q; CHECK: r = b - A x
-        for (int w = blockIdx.x; w < nwork; w += nb) {
+        for (int w = blockIdx.x + nb * ti; w < nwork; w += NG * nb) {
             const int i = wl_inst[w];
             volatile BState* vs = st + i;
-            if (vs->done || vs->mode == 2) continue;
+            const int done = vs->done, mode = vs->mode, par = vs->parity;
+            const double beta = vs->beta;
+            if (done || mode == 2) continue;
             const BInst& I = inst[i];
-            BState* s = st + i;
-            double v;
-            if (vs->mode == 0) {
-                int par = vs->parity;
-                v = apply2d_tile<double, double, MODE_CG, TY, 256>(I.L, wl_c0[w], wl_r0[w], I.cf, I.z, I.q,
-                                                                   I.p[par], I.p[par ^ 1], vs->beta, nullptr, sm);
-                tile_report(v, 0.0, part, w, s, I, [&](double pq, double) {
+            double v[1];
+            if (mode == 0) {
+                v[0] = apply2d_tile<double, double, MODE_CG, TY, TG::NT>(tg, I.L, wl_c0[w], wl_r0[w], I.cf, I.z, I.q,
+                                                                         I.p[par], I.p[par ^ 1], beta, nullptr, sm);
+                tile_report<TY, 1>(tg, rs, v, part, w, st + i, I, [&](const double (&tot)[1], BState* s) {
+                    const double pq = tot[0];
                     if (!(pq > 0.0) || !isfinite(pq)) {
-                        s->done = 1;
+                        s->done = 2;                       // counted in phase D
                         s->status = isfinite(pq) ? STOKES_ERR_BREAKDOWN : STOKES_ERR_NONFINITE;
-                        atomicAdd(&g->ndone, 1);
                     } else {
                         s->alpha = s->rz / pq;
                     }
                 });
             } else {
-                v = apply2d_tile<double, double, MODE_RESID, TY, 256>(I.L, wl_c0[w], wl_r0[w], I.cf, I.x, I.r,
-                                                                      nullptr, nullptr, 0.0, I.b, sm);
-                tile_report(v, 0.0, part, w, s, I, [&](double, double) {});
+                v[0] = apply2d_tile<double, double, MODE_RESID, TY, TG::NT>(tg, I.L, wl_c0[w], wl_r0[w], I.cf, I.x, I.r,
+                                                                            nullptr, nullptr, 0.0, I.b, sm);
+                tile_report<TY, 1>(tg, rs, v, part, w, st + i, I, [&](const double (&)[1], BState*) {});
             }
-            __syncthreads();
+            tg.sync();
         }
-        if (!grid_sync(g, nb)) return;
+        if (!grid_sync(g, nb, bars)) return;
         // ---- phase C (Schwarz): local solves on r_eff = r - alpha q ----------
         if (SW) {
-            for (int k = blockIdx.x; k < npatch; k += nb) {
-                const int i = pl_inst[k];
-                volatile BState* vs = st + i;
-                if (vs->done) continue;
-                const double alpha = vs->mode == 0 ? vs->alpha : 0.0;
-                batched_local_solve(inst[i], pl_patch[k], alpha, Fs, ls, ls, lhb, &lbar, uses, lok, g);
+            // What a patch's copy needs is read a patch ahead, where the patch is
+            // found in the list two ahead: no wait of a patch's own is spent on it.
+            const int step = 2 * nb;
+            int k = blockIdx.x + nb * gi, ki = -1, kp = 0;
+            auto find = [&]() {
+                ki = -1;
+                if (k < npatch) { ki = pl_inst[k]; kp = pl_patch[k]; }
+                k += step;
+            };
+            auto read = [&]() {
+                PatchRef c{ki, kp, 0, 0, false};
+                if (ki >= 0) {
+                    const SchwarzPlan& P = inst[ki].sw;
+                    c.on = !((volatile BState*)st + ki)->done;
+                    c.n = P.nloc[kp];
+                    c.corner = P.corner[kp];
+                }
+                return c;
+            };
+            find();
+            PatchRef cur = read();
+            if (grp.t == 0 && cur.on) patch_issue(inst[cur.inst], cur, Fs, &lbar[gi]);
+            find();
+            while (copies && cur.inst >= 0) {
+                const PatchRef next = read();
+                find();
+                if (cur.on)
+                    copies = batched_local_solve(grp, inst, st, cur, next, Fs, ls[gi], lraw[gi], lhb[gi], &lbar[gi], uses,
+                                                 lok[gi], g);
+                else if (grp.t == 0 && next.on)
+                    patch_issue(inst[next.inst], next, Fs, &lbar[gi]);
+                cur = next;
             }
-            if (!grid_sync(g, nb)) return;
+            if (!grid_sync(g, nb, bars)) return;
         }
         // ---- phase D: CG: x += alpha p, r -= alpha q; z = M^-1 r; r.z, r.r ---
-        for (int w = blockIdx.x; w < nwork; w += nb) {
+        for (int w = blockIdx.x + nb * ti; w < nwork; w += NG * nb) {
             const int i = wl_inst[w];
             volatile BState* vs = st + i;
-            if (vs->done) continue;
             const BInst& I = inst[i];
-            const bool swi = SW && I.use_sw;
-            BState* s = st + i;
-            const int64_t S = I.L.stride;
-            const int mode = vs->mode;
+            const int done = vs->done, mode = vs->mode, par = vs->parity;
             const double alpha = vs->alpha;
-            const double* pn = I.p[vs->parity ^ 1];
-            double rz = 0.0, rr = 0.0;
-            for (int row = warp; row < TY; row += 8) {
+            if (done) {
+                if (done == 2 && w == I.tb && tg.thread() == 0) { vs->done = 1; atomicAdd(&g->ndone, 1); }
+                continue;
+            }
+            const bool swi = SW && I.use_sw;
+            const int64_t S = I.L.stride;
+            const double* pn = I.p[par ^ 1];
+            double sums[2] = {0.0, 0.0};
+            double &rz = sums[0], &rr = sums[1];
+            for (int row = warp; row < TY; row += TG::NW) {
                 const int c = wl_c0[w] + lane, rw = wl_r0[w] + row;
                 int64_t o = I.L.off(c, rw, 0);
-                for (int f = 0; f < 3; ++f) {
-                    int64_t of = f * S + o;
-                    double r;
-                    if (mode == 0) {
-                        I.x[of] += alpha * pn[of];
-                        r = I.r[of] - alpha * I.q[of];
-                        I.r[of] = r;
-                    } else {
-                        r = I.r[of];
+                double r[3], z[3], x[3];
+#pragma unroll
+                for (int f = 0; f < 3; ++f) r[f] = I.r[f * S + o];
+                if (mode == 0) {
+#pragma unroll
+                    for (int f = 0; f < 3; ++f) {
+                        x[f] = I.x[f * S + o] + alpha * pn[f * S + o];
+                        r[f] = r[f] - alpha * I.q[f * S + o];
                     }
-                    double z = swi ? batched_gather(I, f, c - 1, rw - 1, r) : I.minv[of] * r;
-                    I.z[of] = z;
-                    rz = fma(r, z, rz); rr = fma(r, r, rr);
+                }
+                if (swi) batched_gather(I, c - 1, rw - 1, r, z);
+                else
+#pragma unroll
+                    for (int f = 0; f < 3; ++f) z[f] = I.minv[f * S + o] * r[f];
+                if (mode == 0) {
+#pragma unroll
+                    for (int f = 0; f < 3; ++f) { I.x[f * S + o] = x[f]; I.r[f * S + o] = r[f]; }
+                }
+#pragma unroll
+                for (int f = 0; f < 3; ++f) {
+                    I.z[f * S + o] = z[f];
+                    rz = fma(r[f], z[f], rz); rr = fma(r[f], r[f], rr);
                 }
             }
-            tile_report(warp_sum(rz), warp_sum(rr), part, w, s, I, [&](double trz, double trr) {
+            tile_report<TY, 2>(tg, rs, sums, part, w, st + i, I, [&](const double (&tot)[2], BState* s) {
+                const double trz = tot[0], trr = tot[1];
                 s->rr = trr;
                 if (!isfinite(trr) || !isfinite(trz)) {
                     s->done = 1; s->status = STOKES_ERR_NONFINITE; atomicAdd(&g->ndone, 1); return;
@@ -403,9 +525,9 @@ __global__ void __launch_bounds__(256) k_batched(const BInst* __restrict__ inst,
                     }
                 }
             });
-            __syncthreads();
+            tg.sync();
         }
-        if (!grid_sync(g, nb)) return;
+        if (!grid_sync(g, nb, bars, &ndone)) return;
     }
 }
 

@@ -609,18 +609,14 @@ __global__ void __launch_bounds__(256, 2) k_apply2d_v4(Layout L, const int* __re
 //   y_txz = d_xz txz + a_xz [z_u(q) - z_u(q-1) + z_w(c) - z_w(c-1)]
 //   y_tyz = d_yz tyz + a_yz [z_v(q) - z_v(q-1) + z_w(r) - z_w(r-1)]
 //
-// The kernel streams along z: a CTA (256 threads) owns a unit of 32 x 8
-// slots and zt tile layers (16 planes; 4 where the active tiles are too few
-// to fill the device with deep units) and walks its planes in order, keeping two staged
+// k_apply3d (FP64 vectors; FP32 ones take k_apply3d_rows below) streams along z: a
+// CTA (256 threads) owns a unit of 32 x 8 slots and zt tile layers (16 planes; 4
+// where the active tiles are too few to fill the device with deep units) and walks
+// its planes in order, keeping two staged
 // planes (34 x 10 positions) and two planes of each face direction in
 // shared memory.  Every staged value is loaded once per unit (halo 1.33x in
 // x and y, 1.13x in z), against 2.4 staged positions per output for a
-// 32 x 4 x 4 tile holding all its planes at once (FP32 on a 256^3 box: 0.63
-// of the measured HBM bandwidth against 0.49).  Issuing a plane's own-value
-// and coefficient loads before its staging (one memory round trip per
-// plane, 64 registers, 4 CTAs per SM) measured 0.63 for FP32 and lost for
-// BF16 coefficients (0.47 against 0.57) and FP64; 8 CTAs per SM at 32
-// registers lost too (0.58).  For output plane q the step
+// 32 x 4 x 4 tile holding all its planes at once.  For output plane q the step
 //   1. stages plane q+1 (in CG mode p = z + beta p_old, written to p_new on
 //      the unit's own slots of active tiles),
 //   2. forms z_u(q), z_v(q) (staged planes q, q+1) and z_w(q+1) (planes q,
@@ -638,7 +634,7 @@ template <class T> struct Smem3 {
 };
 
 template <class T, class C, int MODE>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout L, Coef<C> cf, const T* __restrict__ x,
+__global__ void __launch_bounds__(256, 3) k_apply3d(Layout L, Coef<C> cf, const T* __restrict__ x,
                                                                           T* __restrict__ y, ApplyArgs args) {
     using SM = Smem3<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -647,7 +643,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
     const int t = threadIdx.x;
     const int nuy = units_y(L.nty);
     const int u = args.units ? args.units[blockIdx.x] : blockIdx.x;
-    const int zt = args.units ? args.zt : ZT_MAX;   // tile layers per unit
+    const int zt = args.zt;                         // tile layers per unit
     unsigned mask;
     const int ux = u % L.ntx, urest = u / L.ntx, uy = urest % nuy, uz = urest / nuy;
     if (args.umask) {
@@ -676,16 +672,6 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
     const C *a_c = cf.f[0], *a_xy = cf.f[1], *a_xz = cf.f[2], *a_yz = cf.f[3];
     const C *d_c = cf.f[4], *d_xy = cf.f[5], *d_xz = cf.f[6], *d_yz = cf.f[7];
     const C *K_u = cf.f[8], *K_v = cf.f[9], *K_w = cf.f[10];
-    // BF16: a slot's row weights and its diagonal from the arrays in fours
-    // (one 8-byte load each), the face coefficients through L2 only (a warp's
-    // 2-byte loads cover half of a 128-byte line)
-    constexpr bool QD = sizeof(C) == 2;
-    const uint2* __restrict__ qa = cf.qd[0];
-    const uint2* __restrict__ qdg = cf.qd[1];
-    auto ldk = [&](const C* p, int64_t o) -> T {
-        if constexpr (QD) return T(__uint_as_float((uint32_t)__ldcg(reinterpret_cast<const unsigned short*>(p + o)) << 16));
-        else return ld<T, C>(p, o);
-    };
     const T* pold = (const T*)args.pold;
     T* pnew = (T*)args.pnew;
     const T beta = MODE == MODE_CG ? (T)args.sc->beta : T(0);
@@ -717,13 +703,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
 #pragma unroll
                 for (int f = 0; f < 6; ++f) pnew[f * S + o] = v[f];
             }
-            T ac, axy, axz, ayz;
-            if constexpr (QD) {
-                const uint2 w = __ldg(qa + o);
-                ac = T(plo(w.x)); axy = T(phi(w.x)); axz = T(plo(w.y)); ayz = T(phi(w.y));
-            } else {
-                ac = ld<T, C>(a_c, o); axy = ld<T, C>(a_xy, o); axz = ld<T, C>(a_xz, o); ayz = ld<T, C>(a_yz, o);
-            }
+            const T ac = ld<T, C>(a_c, o), axy = ld<T, C>(a_xy, o), axz = ld<T, C>(a_xz, o), ayz = ld<T, C>(a_yz, o);
             st[0][e] = ac * (v[5] - v[0]);
             st[1][e] = ac * (v[5] - v[1]);
             st[2][e] = ac * (v[5] + v[0] + v[1]);
@@ -743,9 +723,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
             if (e < SM::NF) {
                 const int ii = e % SM::FX, jj = e / SM::FX;
                 if (r0 + jj <= L.R) {
-                    k[it][0] = ldk(K_u, L.off(c0 + ii, r0 - 1 + jj, q));
-                    k[it][1] = ldk(K_v, L.off(c0 - 1 + ii, r0 + jj, q));
-                    k[it][2] = ldk(K_w, L.off(c0 - 1 + ii, r0 - 1 + jj, q + 1));
+                    k[it][0] = ld<T, C>(K_u, L.off(c0 + ii, r0 - 1 + jj, q));
+                    k[it][1] = ld<T, C>(K_v, L.off(c0 - 1 + ii, r0 + jj, q));
+                    k[it][2] = ld<T, C>(K_w, L.off(c0 - 1 + ii, r0 - 1 + jj, q + 1));
                 }
             }
         }
@@ -866,15 +846,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
             const T zv_cm = zv_q[fi(tx, ty)], zv_qm = zv_m[fi(tx + 1, ty)];
             const T zw = zw_q[fi(tx + 1, ty + 1)], zw_qp = zw_p[fi(tx + 1, ty + 1)];
             const T zw_cm = zw_q[fi(tx, ty + 1)], zw_rm = zw_q[fi(tx + 1, ty)];
-            T ac, axy, axz, ayz, dc, dxy, dxz, dyz;
-            if constexpr (QD) {
-                const uint2 wa = __ldg(qa + o), wd = __ldg(qdg + o);
-                ac = T(plo(wa.x)); axy = T(phi(wa.x)); axz = T(plo(wa.y)); ayz = T(phi(wa.y));
-                dc = T(plo(wd.x)); dxy = T(phi(wd.x)); dxz = T(plo(wd.y)); dyz = T(phi(wd.y));
-            } else {
-                ac = ld<T, C>(a_c, o); axy = ld<T, C>(a_xy, o); axz = ld<T, C>(a_xz, o); ayz = ld<T, C>(a_yz, o);
-                dc = ld<T, C>(d_c, o); dxy = ld<T, C>(d_xy, o); dxz = ld<T, C>(d_xz, o); dyz = ld<T, C>(d_yz, o);
-            }
+            const T ac = ld<T, C>(a_c, o), axy = ld<T, C>(a_xy, o), axz = ld<T, C>(a_xz, o), ayz = ld<T, C>(a_yz, o);
+            const T dc = ld<T, C>(d_c, o), dxy = ld<T, C>(d_xy, o), dxz = ld<T, C>(d_xz, o), dyz = ld<T, C>(d_yz, o);
             T yv[6];
             if (ac != T(0)) {
                 const T ww = zw - zw_qp;
@@ -920,6 +893,232 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_apply3d(Layout 
     }
 }
 
+// 3D apply with FP32 vectors: the walk of k_apply3d with one
+// thread per staged position (ii, jj) of the 34 x 10: warps 0..7 take the rows of
+// the unit's own slots, 8 and 9 the rows before and after, the last the two halo
+// columns.  A thread loads what belongs to its
+// position straight into registers, a plane ahead, and keeps its own staged values,
+// faces and vector entries there from plane to plane; shared memory carries only
+// what a neighbour reads.
+//
+// What bounds it: the latency of a plane's loads (one step ahead, 22 warps per SM)
+// and two barriers a step.  256^3 box: 348 us = 4.6 TB/s of the 1.58 GB it must
+// move, 0.67 of the measured HBM bandwidth; k_apply3d 406 us (three memory round
+// trips a plane, 18 shared-memory reads per face position where this has 6).  The
+// thin liquid column (238 units of 4 planes): 21.2 -> 18.0 ms for the whole step.
+// Copying planes to shared memory ahead with cp.async lost (445 us: the copies, the
+// reads back and the neighbours' reads fill the shared-memory pipe), and so did
+// asking L2 for the rows three planes ahead (433 us).
+// Arithmetic and summation order are k_apply3d's.
+struct Smem3r {
+    static constexpr int SX = TX + 2, NS = SX * (UY3 + 2), PAD = SX;
+    float U[PAD + NS], V[PAD + NS], N[NS + PAD], Nxz[NS + PAD], Nyz[NS + PAD];
+    float zu[PAD + NS + PAD], zv[PAD + NS + PAD], zw[2][PAD + NS];
+};
+constexpr int NT3R = 32 * (UY3 + 3);             // 352
+
+template <class C, int MODE>
+__global__ void __launch_bounds__(NT3R, 2)
+    k_apply3d_rows(Layout L, Coef<C> cf, const float* __restrict__ x, float* __restrict__ y, ApplyArgs args) {
+    using SM = Smem3r;
+    __shared__ SM sm;
+    const int nuy = units_y(L.nty);
+    const int u = args.units ? args.units[blockIdx.x] : blockIdx.x;
+    const int zt = args.zt;
+    const int ux = u % L.ntx, urest = u / L.ntx, uy = urest % nuy, uz = urest / nuy;
+    unsigned mask;
+    if (args.umask) {
+        mask = args.umask[u];
+    } else {
+        mask = 0;
+        for (int dz = 0; dz < zt; ++dz)
+            for (int dy = 0; dy < 2; ++dy)
+                if (2 * uy + dy < L.nty && zt * uz + dz < L.ntz) mask |= 1u << (dy + 2 * dz);
+    }
+    const int c0 = ux * TX, r0 = uy * UY3, q0 = uz * zt * TZ3;
+    const int64_t S = L.stride, PS = (int64_t)L.R * L.P;
+    const float* __restrict__ pold = (const float*)args.pold;
+    const float* __restrict__ b = (const float*)args.b;
+    float* __restrict__ pnew = (float*)args.pnew;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool row = w < UY3 + 2;                // a row's slots; else lane: side + 2 row
+    const int jj = row ? (w < UY3 ? w + 1 : w == UY3 ? 0 : UY3 + 1) : min(lane >> 1, UY3 + 1), ii = row ? lane + 1 : (lane & 1) * (TX + 1);
+    const int e = jj * SM::SX + ii, r = r0 - 1 + jj;
+    const bool inner = row && jj >= 1 && jj <= UY3;
+    // rows past the padded rows are zeros (see k_apply3d); no loads for what no
+    // output needs
+    const bool on = (row || lane < 2 * (UY3 + 2)) && r <= L.R;
+    const bool on_u = on && ii >= 1 && jj <= UY3 && r < L.R, on_v = on && ii <= TX && jj >= 1,
+               on_w = on && ii <= TX && jj <= UY3 && r < L.R;
+    const int64_t o0 = L.off(c0 - 1 + ii, r, 0);
+    int dz_end = 0;
+    for (int dz = 0; dz < zt; ++dz)
+        if ((mask >> (2 * dz)) & 3u) dz_end = dz + 1;
+    const int q_end = q0 + TZ3 * dz_end;
+    auto active = [&](int q) { return inner && ((mask >> ((jj - 1) / TY3 + 2 * ((q - q0) / TZ3))) & 1u) != 0; };
+
+    // group g: x, p_old and a of plane g + 1, K_u, K_v and d (and b) of plane g, K_w of plane g + 1
+    // (BF16: a slot's row weights and its diagonal from the arrays in fours)
+    constexpr bool QD = sizeof(C) == 2;
+    struct Four { float f[QD ? 1 : 4]; uint2 w; };
+    float nx[6], np[6], nb[6];
+    Four na, nd;
+    C nk[3];
+    auto load4 = [&](Four& d, int f0, int64_t o) {
+        if constexpr (QD) d.w = __ldg(cf.qd[f0 / 4] + o);
+        else
+#pragma unroll
+            for (int f = 0; f < 4; ++f) d.f[f] = __ldg(cf.f[f0 + f] + o);
+    };
+    auto zero4 = [](Four& d) {
+        if constexpr (QD) d.w = make_uint2(0u, 0u);
+        else
+#pragma unroll
+            for (int f = 0; f < 4; ++f) d.f[f] = 0.f;
+    };
+    auto get4 = [](const Four& d, float (&v)[4]) {
+        if constexpr (QD) {
+            v[0] = plo(d.w.x); v[1] = phi(d.w.x); v[2] = plo(d.w.y); v[3] = phi(d.w.y);
+        } else
+#pragma unroll
+            for (int f = 0; f < 4; ++f) v[f] = d.f[f];
+    };
+    auto load_x = [&](int q) {
+        const int64_t o = o0 + q * PS;
+#pragma unroll
+        for (int f = 0; f < 6; ++f) {
+            nx[f] = on ? __ldg(x + f * S + o) : 0.f;
+            if (MODE == MODE_CG) np[f] = on ? __ldg(pold + f * S + o) : 0.f;
+        }
+        if (on) load4(na, 0, o);
+        else zero4(na);
+    };
+    auto load_k = [&](int g) {
+        const int64_t o = o0 + g * PS;
+        nk[0] = on_u ? __ldg(cf.f[8] + o) : C(0.f);
+        nk[1] = on_v ? __ldg(cf.f[9] + o) : C(0.f);
+        nk[2] = on_w ? __ldg(cf.f[10] + o + PS) : C(0.f);
+        if (g >= q0 && inner) {
+            load4(nd, 4, o);
+            if (MODE == MODE_RESID)
+#pragma unroll
+                for (int f = 0; f < 6; ++f) nb[f] = __ldg(b + f * S + o);
+        }
+    };
+    Acc<float> acc;
+    if (q_end > q0) {
+        float v0[6], a0[4], v1[6], a1[4], beta = 0.f;
+        load_x(q0 - 1);
+#pragma unroll
+        for (int f = 0; f < 6; ++f) v0[f] = nx[f], v1[f] = MODE == MODE_CG ? np[f] : 0.f;
+        get4(na, a0);
+        load_x(q0);
+        load_k(q0 - 1);
+        if (MODE == MODE_CG) {
+            if (args.sc->done) return;
+            beta = (float)args.sc->beta;
+#pragma unroll
+            for (int f = 0; f < 6; ++f) v0[f] = v0[f] + beta * v1[f];
+        }
+        float zu_m = 0.f, zv_m = 0.f, zw0 = 0.f;
+        // (the products are rounded: a difference of two must not take one in unrounded)
+        float W0 = __fmul_rn(a0[0], v0[5] + v0[0] + v0[1]), Nxz0 = __fmul_rn(a0[2], v0[3]), Nyz0 = __fmul_rn(a0[3], v0[4]);
+        for (int g = q0 - 1; g < q_end; ++g) {
+            // own values of plane g + 1; the next group's loads
+            float d[4], bb[6], k[3];
+#pragma unroll
+            for (int f = 0; f < 6; ++f) v1[f] = MODE == MODE_CG ? nx[f] + beta * np[f] : nx[f];
+            get4(na, a1);
+            get4(nd, d);
+#pragma unroll
+            for (int f = 0; f < 3; ++f) k[f] = (float)nk[f];
+            if (MODE == MODE_RESID)
+#pragma unroll
+                for (int f = 0; f < 6; ++f) bb[f] = nb[f];
+            if (g + 1 < q_end) {
+                load_x(g + 2);
+                load_k(g + 1);
+                if (MODE == MODE_CG && active(g + 1)) {
+#pragma unroll
+                    for (int f = 0; f < 6; ++f) pnew[f * S + o0 + (g + 1) * PS] = v1[f];
+                }
+            }
+            // staged values a neighbour reads: U, V, Nxy of plane g, Nxz, Nyz of plane g + 1
+            const float U = __fmul_rn(a0[0], v0[5] - v0[0]), V = __fmul_rn(a0[0], v0[5] - v0[1]), N = __fmul_rn(a0[1], v0[2]);
+            const float W1 = __fmul_rn(a1[0], v1[5] + v1[0] + v1[1]), Nxz1 = __fmul_rn(a1[2], v1[3]), Nyz1 = __fmul_rn(a1[3], v1[4]);
+            if (row || lane < 2 * (UY3 + 2)) {
+                sm.U[SM::PAD + e] = U;
+                sm.V[SM::PAD + e] = V;
+                sm.N[e] = N;
+                sm.Nxz[e] = Nxz1;
+                sm.Nyz[e] = Nyz1;
+            }
+            __syncthreads();
+            const float zu = __fmul_rn(k[0], (U - sm.U[SM::PAD + e - 1]) + (N - sm.N[e + SM::SX]) + (Nxz0 - Nxz1));
+            const float zv = __fmul_rn(k[1], (V - sm.V[SM::PAD + e - SM::SX]) + (N - sm.N[e + 1]) + (Nyz0 - Nyz1));
+            const float zw1 = __fmul_rn(k[2], (W1 - W0) + (Nxz1 - sm.Nxz[e + 1]) + (Nyz1 - sm.Nyz[e + SM::SX]));
+            if (row || lane < 2 * (UY3 + 2)) {
+                sm.zu[SM::PAD + e] = zu;
+                sm.zv[SM::PAD + e] = zv;
+                sm.zw[(g + 1) & 1][SM::PAD + e] = zw1;
+            }
+            __syncthreads();
+            if (g >= q0 && active(g)) {
+                const int64_t o = o0 + g * PS;
+                const float zu_cp = sm.zu[SM::PAD + e + 1], zu_rm = sm.zu[SM::PAD + e - SM::SX];
+                const float zv_rp = sm.zv[SM::PAD + e + SM::SX], zv_cm = sm.zv[SM::PAD + e - 1];
+                const float zw_cm = sm.zw[g & 1][SM::PAD + e - 1], zw_rm = sm.zw[g & 1][SM::PAD + e - SM::SX];
+                const float zw = zw0, zw_qp = zw1, zu_qm = zu_m, zv_qm = zv_m;
+                const float ac = a0[0], axy = a0[1], axz = a0[2], ayz = a0[3];
+                const float dc = d[0], dxy = d[1], dxz = d[2], dyz = d[3];
+                float yv[6];
+                if (ac != 0.f) {
+                    const float ww = zw - zw_qp;
+                    yv[5] = ac * ((zu - zu_cp) + (zv - zv_rp) + ww);
+                    yv[0] = fmaf(ac, (zu_cp - zu) + ww, dc * (v0[0] + 0.5f * v0[1]));
+                    yv[1] = fmaf(ac, (zv_rp - zv) + ww, dc * (v0[1] + 0.5f * v0[0]));
+                } else {
+                    yv[5] = v0[5]; yv[0] = v0[0]; yv[1] = v0[1];
+                }
+                yv[2] = fmaf(axy, (zu - zu_rm) + (zv - zv_cm), dxy * v0[2]);
+                yv[3] = fmaf(axz, (zu - zu_qm) + (zw - zw_cm), dxz * v0[3]);
+                yv[4] = fmaf(ayz, (zv - zv_qm) + (zw - zw_rm), dyz * v0[4]);
+                if (MODE == MODE_RESID)
+#pragma unroll
+                    for (int f = 0; f < 6; ++f) yv[f] = bb[f] - yv[f];
+#pragma unroll
+                for (int f = 0; f < 6; ++f) y[f * S + o] = yv[f];
+                if (MODE == MODE_RESID) {
+#pragma unroll
+                    for (int f = 0; f < 6; ++f) acc.add(yv[f], yv[f]);
+                } else if (MODE == MODE_CG) {
+#pragma unroll
+                    for (int f = 0; f < 6; ++f) acc.add(v0[f], yv[f]);
+                }
+            }
+            zu_m = zu; zv_m = zv; zw0 = zw1;
+            W0 = W1; Nxz0 = Nxz1; Nyz0 = Nyz1;
+#pragma unroll
+            for (int f = 0; f < 6; ++f) v0[f] = v1[f];
+#pragma unroll
+            for (int f = 0; f < 4; ++f) a0[f] = a1[f];
+        }
+    } else if (MODE == MODE_CG && args.sc->done) {
+        return;
+    }
+    if (MODE != MODE_PLAIN) {
+        CgScalars* sc = args.sc;
+        const Acc<float> sums[1] = {acc};
+        block_sums<float, 1>(sums, args.partial, args.counter, gridDim.x, [&](const double (&tots)[1]) {
+            const double tot = tots[0];
+            if (MODE == MODE_RESID) { sc->rr = tot; return; }
+            sc->pq = tot;
+            if (!(tot > 0.0) || !isfinite(tot)) { sc->done = 1; sc->status = (isfinite(tot) ? STOKES_ERR_BREAKDOWN : STOKES_ERR_NONFINITE); }
+            else sc->alpha = sc->rz / tot;
+        });
+    }
+}
+
 // CTAs that fit on the device at once for a kernel (cached per device): the
 // persistent kernels launch min(tiles, this) CTAs.
 static int resident_ctas(const void* fn, int threads, size_t smem, int* cache) {
@@ -935,11 +1134,18 @@ static int resident_ctas(const void* fn, int threads, size_t smem, int* cache) {
     return cache[dev];
 }
 
+static int sm_count() {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return std::max(1, n);
+}
+
 template <class T, class C, int MODE>
 static cudaError_t launch_mode(const Layout& L, const int* tiles, int ntiles, const Coef<C>& cf, const T* x, T* y,
                                const ApplyArgs& a, cudaStream_t s) {
     if (ntiles <= 0) return cudaSuccess;
-    static int cache2[16], cache3[16];
+    static int cache2[16];
     if (L.dim == 2) {
         // FP64 vectors: one slot per thread, software-pipelined over the tiles
         // (bound by the FP64 pipe).  In the CG loop the unconstrained build is
@@ -970,11 +1176,27 @@ static cudaError_t launch_mode(const Layout& L, const int* tiles, int ntiles, co
     } else {
         // 3D: one CTA per unit (32 x 8 slots, 16 planes), over the active
         // units (an apply over the active tiles needs the unit list) or all
-        (void)cache3;
         if (tiles && !a.units) return cudaErrorInvalidValue;
         if (sizeof(C) == 2 && !cf.qd[0]) return cudaErrorInvalidValue;   // BF16 reads the arrays in fours
-        const int nu = tiles ? a.nunits : L.ntx * units_y(L.nty) * units_z(L.ntz, ZT_MAX);
-        if (nu > 0) k_apply3d<T, C, MODE><<<nu, 256, sizeof(Smem3<T>), s>>>(L, cf, x, y, a);
+        ApplyArgs b = a;
+        if (!a.units) {
+            // the whole grid: units of 16 planes (1.13 planes staged per plane of
+            // output), of 8 or 4 where those would be fewer than two per SM (64^3,
+            // 135 units of 16: FP32 34.9 -> 18.8 us, FP64 119 -> 86; up to three per
+            // SM lost for FP64 boxes that are bound by arithmetic: 129 x 97 x 65, 325
+            // units, 209 -> 220)
+            b.zt = ZT_MAX;
+            if (MODE == MODE_PLAIN) {
+                const int two = 2 * sm_count();
+                while (b.zt > 1 && L.ntx * units_y(L.nty) * units_z(L.ntz, b.zt) < two) b.zt /= 2;
+            }
+        }
+        const int nu = tiles ? a.nunits : L.ntx * units_y(L.nty) * units_z(L.ntz, b.zt);
+        if constexpr (sizeof(T) == 4) {
+            if (nu > 0) k_apply3d_rows<C, MODE><<<nu, NT3R, 0, s>>>(L, cf, x, y, b);
+        } else {
+            if (nu > 0) k_apply3d<T, C, MODE><<<nu, 256, sizeof(Smem3<T>), s>>>(L, cf, x, y, b);
+        }
     }
     return cudaGetLastError();
 }
@@ -1001,8 +1223,6 @@ static void set_attr3() {
 // process and device, before any launch or graph capture).
 void apply_set_attributes() {
     set_attr3<double, double>();
-    set_attr3<float, float>();
-    set_attr3<float, __nv_bfloat16>();
 }
 
 template cudaError_t launch_apply_mode<double, double>(const Layout&, const int*, int, const Coef<double>&,

@@ -68,14 +68,15 @@ template <int Q> struct BlockSumSmem {
     bool last;
 };
 
-// The block's sums of the threads' accumulators into partial[Q blockIdx.x + q];
+// The block's sums of its first 256 threads' accumulators into partial[Q blockIdx.x + q];
 // the last block to finish adds up all blocks and calls fin(totals) in one
-// thread.  Every thread of the 256 calls it, once per kernel.
+// thread.  Every thread of the block calls it, once per kernel.
 template <class T, int Q, class Fin>
 __device__ __forceinline__ void block_sums(const Acc<T> (&acc)[Q], double* partial, unsigned* counter, int nblocks, Fin fin) {
     __shared__ BlockSumSmem<Q> sm;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    if constexpr (sizeof(T) == 4) {
+    if (w >= 8) {
+    } else if constexpr (sizeof(T) == 4) {
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             const float2 v = warp_ff(acc[q].hi, acc[q].lo);
@@ -107,7 +108,7 @@ __device__ __forceinline__ void block_sums(const Acc<T> (&acc)[Q], double* parti
     __syncthreads();
     if (!sm.last) return;
     __threadfence();
-    if (32 * w < nblocks) {
+    if (w < 8 && 32 * w < nblocks) {
         double v[Q];
 #pragma unroll
         for (int q = 0; q < Q; ++q) v[q] = t < nblocks ? ((volatile double*)partial)[Q * t + q] : 0.0;

@@ -302,7 +302,11 @@ __global__ void __launch_bounds__(128, 15) k_schwarz_gemv(Layout L, SchwarzPlan 
     __shared__ __align__(8) unsigned long long bar;
     __shared__ int ok_s;
     const int t = threadIdx.x;
-    const int p = blockIdx.x;
+    // Factors that do not fit in L2 are walked there and back from one step to the
+    // next: the part L2 holds at a step's end is what the next one starts with
+    // (1024^2 bumps, 229 MB of factors: the whole step 368 -> 360 ms; keeping any
+    // share of them in L2 by the normal or the evict-last policy made it slower)
+    const int p = P.evict_first && (sc->iter & 1) ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
     const uint32_t b_addr = smem_u32(&bar);
     // the patch's size and corner and the solve's scalars are loaded together
     // (one memory round trip before the copy starts)

@@ -52,18 +52,21 @@ __global__ void k_schwarz_mark(Layout L, DevArrays D, int npx, int npy, int* fla
 // issued in parallel (activity flags, then the coefficients of the faces
 // touching the patch, staged in shared memory); each thread accumulates one
 // row, faces in a fixed order, so the local matrices are reproducible bit for
-// bit.  Dynamic smem: the FP64 matrix (PMAX^2 doubles), whose upper half
-// later holds the scaled FP32 matrix and whose lower half the inverse factor
-// X = L^-1, then the diagonal scaling: about 94 KB, two CTAs per SM.
+// bit.  Dynamic smem: the FP64 matrix (PMAX^2 doubles), where the scaled FP32
+// entries then take the low halves of their slots and the inverse factor X = L^-1
+// comes last, then the diagonal scaling: about 94 KB, two CTAs per SM.
+// FP64 instructions and the factorisation's serial chain bound it.  A wave of 304
+// patches took 296 us when each face's rows were found by searching (one lane of a
+// warp at work at a time), every entry was rotated and converted, and the
+// factorisation ran in shared memory with five barriers a column.  Now 1024^2
+// bumps (17,645 patches) 17.9 -> 7.0 ms, a jet of 150^2 cells 296 -> 120 us.
 constexpr int SW_NFACE = 2 * (PR + 2) * (PR + 2);   // faces of both directions around a patch
 constexpr int SW_SETUP_SMEM = PMAX * PMAX * 8 + PMAX * 4;
 __global__ void __launch_bounds__(256) k_schwarz_setup(Layout L, DevArrays D, const double* coef, SchwarzPlan P) {
     extern __shared__ __align__(16) double smd[];
     double* Ad = smd;                                        // n x n (row-major, stride PMAX), FP64
-    float* A = reinterpret_cast<float*>(smd) + PMAX * PMAX;  // upper half: scaled copy, FP32
-    float* X = reinterpret_cast<float*>(smd);                // lower half: L^-1
     float* sc = reinterpret_cast<float*>(smd + PMAX * PMAX); // 1/sqrt(diag)
-    __shared__ short map[PMAX];
+    __shared__ short map[PMAX], pos_of[PMAX];                // local index by position, and back
     __shared__ unsigned ballots[4];
     __shared__ double dd[PMAX];                              // 1/sqrt(diag) in FP64, 0 if not positive
     __shared__ double fK[SW_NFACE], fb[SW_NFACE][6];
@@ -93,6 +96,7 @@ __global__ void __launch_bounds__(256) k_schwarz_setup(Layout L, DevArrays D, co
         for (int q = 0; q < w; ++q) before += __popc(ballots[q]);
         before += __popc(ballots[w] & ((1u << lane) - 1u));
         map[t] = act ? (short)before : (short)-1;
+        if (act) pos_of[before] = (short)t;
         P.lmap[(int64_t)p * PMAX + t] = map[t];
     }
     if (t == 0) P.nloc[p] = n;
@@ -139,53 +143,81 @@ __global__ void __launch_bounds__(256) k_schwarz_setup(Layout L, DevArrays D, co
     }
     __syncthreads();
     // 3. row r of A_p by thread r: the stress diagonal C, then K_f b_f b_f^T
-    // of every face containing r, faces in order (each entry sums the same
+    // of the four faces containing r, faces in order (each entry sums the same
     // terms in the same order whichever thread owns it: reproducible bit for
-    // bit)
+    // bit).  A cell's unknowns are in its own faces, a node's txy in the u faces
+    // below and above it and the v faces left and right; all threads walk their
+    // four at once (FP64 instructions cost a warp the same for one lane as for 32).
+    constexpr int FW = PR + 2;
     if (t < n) {
         double* row = Ad + (int64_t)t * PMAX;
-        int pos = -1;                     // position (field, ring row, ring column) of unknown t
-        for (int e = 0; e < PMAX; ++e)
-            if (map[e] == t) { pos = e; break; }
-        const int f = pos / (PR * PR), cell = pos % (PR * PR);
-        if (f < 2) row[t] += (f == 0 ? d_c : d_n)[L.off(a0 + cell % PR + 1, b0 + cell / PR + 1, 0)];
-        for (int fc = 0; fc < SW_NFACE; ++fc) {
+        const int pos = pos_of[t];
+        const int f = pos / (PR * PR), cell = pos % (PR * PR), ii = cell % PR, jj = cell / PR;
+        if (f < 2) row[t] += (f == 0 ? d_c : d_n)[L.off(a0 + ii + 1, b0 + jj + 1, 0)];
+        for (int s = 0; s < 4; ++s) {
+            const int dir = s >> 1, odd = s & 1;
+            int fi = ii, fj = jj, q;
+            if (f == 1) {
+                if (!odd) { (dir == 0 ? fj : fi) -= 1; }
+                q = odd ? 4 : 5;
+            } else {
+                if (odd) { (dir == 0 ? fi : fj) += 1; }
+                q = (odd ? 0 : 2) + (f == 2 ? 1 : 0);
+            }
+            const int fc = (dir * FW + fj + 1) * FW + fi + 1;
             const double K = fK[fc];
             if (K == 0.0) continue;
-            for (int q = 0; q < 6; ++q) {
-                if (fidx[fc][q] != t) continue;
-                const double kb = K * fb[fc][q];
-                for (int c = 0; c < 6; ++c) {
-                    const int ic = fidx[fc][c];
-                    if (ic >= 0) row[ic] += kb * fb[fc][c];
-                }
+            const double kb = K * fb[fc][q];
+            for (int c = 0; c < 6; ++c) {
+                const int ic = fidx[fc][c];
+                if (ic >= 0) row[ic] += kb * fb[fc][c];
             }
         }
     }
     __syncthreads();
-    // 5. Q A_p Q with Q the symmetric orthogonal pair rotation (rows, then columns)
+    // 5. Q A_p Q with Q the symmetric orthogonal pair rotation (rows, then
+    // columns), on the entries that can be nonzero: a cell couples to itself and
+    // its four neighbours (both fields) and to its four nodes, a node to its four
+    // cells, itself and its four neighbours.  (dense: 3888 pairs a pass, here 504)
+    auto at = [&](int f, int ii, int jj) -> int {
+        return ii < 0 || jj < 0 || ii >= PR || jj >= PR ? -1 : (int)map[(f * PR + jj) * PR + ii];
+    };
+    auto star = [](int k, int& ii, int& jj) {          // the point itself, left, right, below, above
+        ii += (k == 2) - (k == 1);
+        jj += (k == 4) - (k == 3);
+    };
     constexpr double H = 0.70710678118654752440;
-    for (int e = t; e < PR * PR * n; e += 256) {
-        int cell = e / n, c = e % n;
-        int kt = map[cell], kp = map[2 * PR * PR + cell];
+    for (int e = t; e < PR * PR * 14; e += 256) {
+        const int cell = e / 14, k = e % 14;
+        const int kt = map[cell], kp = map[2 * PR * PR + cell];
         if (kt < 0 || kp < 0) continue;
-        double a = Ad[kt * PMAX + c], b = Ad[kp * PMAX + c];
+        int ii = cell % PR, jj = cell / PR;
+        if (k < 10) star(k % 5, ii, jj);
+        else ii += (k - 10) & 1, jj += (k - 10) >> 1;
+        const int c = at(k < 5 ? 0 : k < 10 ? 2 : 1, ii, jj);
+        if (c < 0) continue;
+        const double a = Ad[kt * PMAX + c], b = Ad[kp * PMAX + c];
         Ad[kt * PMAX + c] = (a + b) * H;
         Ad[kp * PMAX + c] = (a - b) * H;
     }
     __syncthreads();
-    for (int e = t; e < PR * PR * n; e += 256) {
-        int cell = e / n, r = e % n;
-        int kt = map[cell], kp = map[2 * PR * PR + cell];
+    for (int e = t; e < PR * PR * 14; e += 256) {
+        const int cell = e / 14, k = e % 14;
+        const int kt = map[cell], kp = map[2 * PR * PR + cell];
         if (kt < 0 || kp < 0) continue;
-        double a = Ad[r * PMAX + kt], b = Ad[r * PMAX + kp];
+        int ii = cell % PR, jj = cell / PR;
+        if (k < 10) star(k % 5, ii, jj);
+        else ii += (k - 10) & 1, jj += (k - 10) >> 1;
+        const int r = at(k < 5 ? 0 : k < 10 ? 2 : 1, ii, jj);
+        if (r < 0) continue;
+        const double a = Ad[r * PMAX + kt], b = Ad[r * PMAX + kp];
         Ad[r * PMAX + kt] = (a + b) * H;
         Ad[r * PMAX + kp] = (a - b) * H;
     }
     __syncthreads();
-    // 6. unit-diagonal scaling (FP64, then rounded to FP32).  The FP32 row r
-    // lands on FP64 rows >= r of the same buffer, so rows are converted from
-    // the last down, a block of rows at a time (read all, barrier, write all).
+    // 6. unit-diagonal scaling (FP64, then rounded to FP32), on the same entries:
+    // the FP32 value takes the low half of its FP64 slot (an entry that cannot be
+    // nonzero is a zero there already)
     // (FP64 divisions and square roots are slow on this part: one per row)
     for (int k = t; k < n; k += 256) {
         const double d = Ad[k * PMAX + k];
@@ -193,72 +225,95 @@ __global__ void __launch_bounds__(256) k_schwarz_setup(Layout L, DevArrays D, co
         sc[k] = d > 0.0 ? (float)dd[k] : 1.f;
     }
     __syncthreads();
-    constexpr int CONV_ROWS = 16;
-    for (int r1 = n; r1 > 0; r1 -= CONV_ROWS) {
-        const int r0 = max(r1 - CONV_ROWS, 0);
-        float v[(CONV_ROWS * PMAX + 255) / 256];
-#pragma unroll
-        for (int q = 0; q < (CONV_ROWS * PMAX + 255) / 256; ++q) {
-            const int e = t + 256 * q, r = r0 + e / PMAX, c = e % PMAX;
-            v[q] = 0.f;
-            if (r < r1 && c < n) {
-                const double sr = dd[r], scc = dd[c];
-                v[q] = (sr > 0.0 && scc > 0.0) ? (float)(Ad[r * PMAX + c] * sr * scc) : (r == c ? 1.f : 0.f);
-            }
+    for (int e = t; e < n * 14; e += 256) {
+        const int r = e / 14, k = e % 14, pos = pos_of[r];
+        const int f = pos / (PR * PR), cell = pos % (PR * PR);
+        int ii = cell % PR, jj = cell / PR, fc;
+        if (f != 1) {
+            if (k < 10) star(k % 5, ii, jj);
+            else ii += (k - 10) & 1, jj += (k - 10) >> 1;
+            fc = k < 5 ? 0 : k < 10 ? 2 : 1;
+        } else if (k < 8) {
+            ii -= k & 1, jj -= (k >> 1) & 1;
+            fc = k < 4 ? 0 : 2;
+        } else {
+            if (k == 13) continue;
+            star(k - 8, ii, jj);
+            fc = 1;
         }
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < (CONV_ROWS * PMAX + 255) / 256; ++q) {
-            const int e = t + 256 * q, r = r0 + e / PMAX, c = e % PMAX;
-            if (r < r1 && c < n) A[r * PMAX + c] = v[q];
-        }
-        __syncthreads();
-    }
-    // 7. Cholesky (lower, in place, FP32).  Column k is copied to colk once
-    // scaled; the trailing update runs on a 16 x 16 thread grid (thread
-    // (tr, tc): rows k+1+tr+16i, columns k+1+tc+16j <= row), lower triangle only
-    __shared__ float colk[PMAX];
-    const int tr = t >> 4, tc = t & 15;
-    for (int k = 0; k < n; ++k) {
-        if (t == 0) {
-            float d = A[k * PMAX + k];
-            A[k * PMAX + k] = d > 1e-12f ? sqrtf(d) : 1.f;    // a vanishing pivot is replaced (robust, still SPD)
-        }
-        __syncthreads();
-        const float piv = A[k * PMAX + k];
-        for (int r = k + 1 + t; r < n; r += 256) {
-            const float v = A[r * PMAX + k] / piv;
-            A[r * PMAX + k] = v;
-            colk[r] = v;
-        }
-        __syncthreads();
-        for (int r = k + 1 + tr; r < n; r += 16) {
-            const float lr = colk[r];
-            float* Ar = A + r * PMAX;
-            for (int c = k + 1 + tc; c <= r; c += 16) Ar[c] -= lr * colk[c];
-        }
-        __syncthreads();
-    }
-    // 8. X = L^-1 by forward elimination on the identity, all columns at
-    // once: row k is final once divided by L_kk, then eliminated from the
-    // rows below (thread (tr, tc): rows k+1+tr+16i, columns tc+16j <= k)
-    for (int e = t; e < n * PMAX; e += 256) {
-        const int r = e / PMAX, c = e - r * PMAX;
-        if (c < n) X[e] = r == c ? 1.f : 0.f;
+        const int c = at(fc, ii, jj);
+        if (c < 0 || c > r) continue;              // the factorisation reads the lower triangle
+        const double sr = dd[r], scc = dd[c];
+        const float v = (sr > 0.0 && scc > 0.0) ? (float)(Ad[r * PMAX + c] * sr * scc) : (r == c ? 1.f : 0.f);
+        *reinterpret_cast<float2*>(&Ad[r * PMAX + c]) = make_float2(v, 0.f);
     }
     __syncthreads();
-    for (int k = 0; k < n; ++k) {
-        const float inv = 1.f / A[k * PMAX + k];
-        for (int c = t; c <= k; c += 256) X[k * PMAX + c] *= inv;
-        __syncthreads();
-        const float* Xk = X + k * PMAX;
-        for (int r = k + 1 + tr; r < n; r += 16) {
-            const float lr = A[r * PMAX + k];
-            float* Xr = X + r * PMAX;
-            for (int c = tc; c <= k; c += 16) Xr[c] -= lr * Xk[c];
+    // 7. Cholesky (lower, FP32) and X = L^-1 by forward elimination on the
+    // identity, in one loop over the columns, both matrices in registers: thread
+    // (tr, tc) of the 16 x 16 grid holds rows tr + 16 i and columns tc + 16 j,
+    // j <= i.  At step k the 16 threads of column k (a half warp) scale it, those of
+    // row k of X publish it, and after one barrier everyone updates the trailing
+    // triangle and the rows of X below.
+    constexpr int NB = (PMAX + 15) / 16, NE = NB * (NB + 1) / 2;
+    __shared__ float colk[2][16 * NB], rowk[2][16 * NB], pivk[2];
+    const int tr = t & 15, tc = t >> 4;
+    float av[NE], xv[NE];
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+#pragma unroll
+        for (int j = 0; j <= i; ++j) {
+            const int r = tr + 16 * i, c = tc + 16 * j;
+            av[i * (i + 1) / 2 + j] = r < n && c <= r ? reinterpret_cast<const float2*>(Ad)[r * PMAX + c].x : 0.f;
+            xv[i * (i + 1) / 2 + j] = r == c ? 1.f : 0.f;
         }
-        __syncthreads();
-    }
+#pragma unroll
+    for (int jb = 0; jb < NB; ++jb)
+        for (int kk = 0; kk < 16; ++kk) {
+            const int k = 16 * jb + kk, buf = kk & 1;
+            if (k >= n) break;
+            if (tc == kk) {
+                const float d = __shfl_sync(0xffffu << (lane & 16), av[jb * (jb + 1) / 2 + jb], kk, 16);
+                const float piv = d > 1e-12f ? sqrtf(d) : 1.f;    // a vanishing pivot is replaced (robust, still SPD)
+                if (tr == kk) pivk[buf] = piv;
+#pragma unroll
+                for (int i = jb; i < NB; ++i)
+                    if (16 * i < n && (i > jb || tr > kk)) colk[buf][tr + 16 * i] = av[i * (i + 1) / 2 + jb] / piv;
+            }
+            if (tr == kk)
+#pragma unroll
+                for (int j = 0; j <= jb; ++j) rowk[buf][tc + 16 * j] = xv[jb * (jb + 1) / 2 + j];
+            __syncthreads();
+            const float inv = 1.f / pivk[buf];
+            float xk[NB], ck[NB];
+#pragma unroll
+            for (int j = 0; j <= jb; ++j) {
+                xk[j] = rowk[buf][tc + 16 * j] * inv;
+                if (tr == kk && (j < jb || tc <= kk)) xv[jb * (jb + 1) / 2 + j] = xk[j];
+            }
+#pragma unroll
+            for (int j = jb; j < NB; ++j) ck[j] = 16 * j < n && (j > jb || tc > kk) ? colk[buf][tc + 16 * j] : 0.f;
+#pragma unroll
+            for (int i = jb; i < NB; ++i) {
+                if (16 * i >= n || (i == jb && tr <= kk)) continue;
+                const float lr = colk[buf][tr + 16 * i];
+#pragma unroll
+                for (int j = jb; j <= i; ++j)
+                    if (j > jb || tc > kk) av[i * (i + 1) / 2 + j] -= lr * ck[j];
+#pragma unroll
+                for (int j = 0; j <= jb; ++j)
+                    if (j < jb || tc <= kk) xv[i * (i + 1) / 2 + j] -= lr * xk[j];
+            }
+        }
+    constexpr int XS = PMAX + 1;                             // an odd stride: no bank conflicts by rows
+    float* X = reinterpret_cast<float*>(smd);                // L^-1 (the FP64 matrix is no longer needed)
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+#pragma unroll
+        for (int j = 0; j <= i; ++j) {
+            const int r = tr + 16 * i, c = tc + 16 * j;
+            if (r < n && c <= r) X[r * XS + c] = xv[i * (i + 1) / 2 + j];
+        }
+    __syncthreads();
     // stored factor: row factors rho_r^2 and the packed FP16 rows X[r][0..r] /
     // rho_r (padded to 16 bytes), and the scaling by position.  The patch
     // operator D^-1/2 X~^T diag(rho^2) X~ D^-1/2 is symmetric positive
@@ -269,7 +324,7 @@ __global__ void __launch_bounds__(256) k_schwarz_setup(Layout L, DevArrays D, co
     if (t < PMAX) {
         float m = 0.f;
         if (t < n)
-            for (int c = 0; c <= t; ++c) m = fmaxf(m, fabsf(X[t * PMAX + c]));
+            for (int c = 0; c <= t; ++c) m = fmaxf(m, fabsf(X[t * XS + c]));
         rho_inv[t] = m > 0.f ? 1.f / m : 0.f;
         reinterpret_cast<float*>(F)[t] = m * m;
     }
@@ -278,7 +333,7 @@ __global__ void __launch_bounds__(256) k_schwarz_setup(Layout L, DevArrays D, co
     const int n8 = (n + 7) / 8 * 8;
     for (int e = t; e < n * n8; e += 256) {
         const int r = e / n8, c = e % n8;
-        if (c < (r / 8 + 1) * 8) Xh[sw_fac_off(r, c, n)] = __float2half_rn(c <= r ? X[r * PMAX + c] * rho_inv[r] : 0.f);
+        if (c < (r / 8 + 1) * 8) Xh[sw_fac_off(r, c, n)] = __float2half_rn(c <= r ? X[r * XS + c] * rho_inv[r] : 0.f);
     }
     for (int e = t; e < PMAX; e += 256) P.scale[(int64_t)p * PMAX + e] = map[e] >= 0 ? sc[map[e]] : 0.f;
 }

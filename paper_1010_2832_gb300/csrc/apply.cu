@@ -593,6 +593,121 @@ __global__ void __launch_bounds__(256, 2) k_apply2d_v4(Layout L, const int* __re
     }
 }
 
+// 2D apply of FP32 vectors over a large whole grid: a warp streams down the rows
+// [r0, r0 + ny) of 120 columns, four columns per lane, the outermost lanes for the
+// halo.  A row's loads go out a row ahead; what the rows share stays in registers
+// and what neighbouring columns share goes by shuffles: no shared memory, no
+// barrier, and every row is read once per chunk of ny rows (plus one on each side).
+// Bound by HBM: 4096^2 box, FP32 120 us = 6.7 TB/s of the 0.80 GB it must move, 0.98
+// of the measured bandwidth (k_apply2d_v4 158 us); BF16 coefficients 103 us against
+// 157.  Products that two positions share are rounded before they are subtracted,
+// and of a sum of two products the first is fused, as in apply2d_tile.
+constexpr int SC2 = 120, SR2 = 8;                // columns of a strip; fewest rows of a chunk
+template <class C> struct Row2 {                 // group s: x, a, K_v of row s; d, K_u of row s - 1
+    float4 x[3], ac, an, dc, dn, ku, kv;
+};
+template <> struct Row2<__nv_bfloat16> {         // pair words: (a_c, a_n), (K_u, K_v) of row s; (d_c, d_n) of row s - 1
+    float4 x[3];
+    uint4 a, k, d;
+};
+template <class C>
+__global__ void __launch_bounds__(256, 2) k_apply2d_stream(Layout L, Coef<C> cf, const float* __restrict__ x,
+                                                           float* __restrict__ y, int strips, int nwarp, int ny) {
+    constexpr bool PAIR = sizeof(C) == 2;
+    const int wi = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (wi >= nwarp) return;
+    const int c = wi % strips * SC2 - 4 + 4 * lane, r0 = wi / strips * ny, r1 = min(r0 + ny, L.R);
+    const bool on = c < L.P + 4;                 // loads stay inside the guards
+    const bool out = lane >= 1 && lane <= 30 && c < L.P;
+    const int64_t S = L.stride, o0 = L.off(c, 0, 0);
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    Row2<C> n;
+    auto ld4 = [&](const float* p, int64_t o) { return __ldg(reinterpret_cast<const float4*>(p + o)); };
+    auto ldp = [&](const uint32_t* p, int64_t o) { return __ldg(reinterpret_cast<const uint4*>(p + o)); };
+    auto load = [&](int s) {
+        if (!on) {
+            n = Row2<C>{};
+            return;
+        }
+        const int64_t o = o0 + (int64_t)s * L.P;
+#pragma unroll
+        for (int f = 0; f < 3; ++f) n.x[f] = ld4(x + f * S, o);
+        if constexpr (PAIR) {
+            n.a = ldp(cf.pr[0], o);
+            n.k = ldp(cf.pr[2], o);
+            n.d = s > r0 ? ldp(cf.pr[1], o - L.P) : make_uint4(0u, 0u, 0u, 0u);
+        } else {
+            n.ac = ld4(cf.f[0], o);
+            n.an = ld4(cf.f[1], o);
+            n.kv = ld4(cf.f[5], o);
+            n.ku = s >= r0 ? ld4(cf.f[4], o - L.P) : zero;
+            n.dc = s > r0 ? ld4(cf.f[2], o - L.P) : zero;
+            n.dn = s > r0 ? ld4(cf.f[3], o - L.P) : zero;
+        }
+    };
+    // of row s - 1: vector entries, row weights, U(c) - U(c - 1), V, N, z_v; z_u of row s - 2
+    float tx[4] = {}, ty[4] = {}, pr[4] = {}, ac[4] = {}, an[4] = {}, du[4] = {}, V[4] = {}, N[4] = {}, zv[4] = {}, zm[4] = {};
+    float kup[4] = {};                           // BF16: K_u of row s - 1
+    load(r0 - 1);
+    for (int s = r0 - 1; s <= r1; ++s) {
+        float x0[4], x1[4], x2[4], a0[4], a1[4], d0[4], d1[4], ku[4], kv[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            x0[i] = f4(n.x[0], i); x1[i] = f4(n.x[1], i); x2[i] = f4(n.x[2], i);
+            if constexpr (PAIR) {
+                a0[i] = plo(u4(n.a, i)); a1[i] = phi(u4(n.a, i));
+                d0[i] = plo(u4(n.d, i)); d1[i] = phi(u4(n.d, i));
+                ku[i] = kup[i]; kup[i] = plo(u4(n.k, i)); kv[i] = phi(u4(n.k, i));
+            } else {
+                a0[i] = f4(n.ac, i); a1[i] = f4(n.an, i);
+                d0[i] = f4(n.dc, i); d1[i] = f4(n.dn, i);
+                ku[i] = f4(n.ku, i); kv[i] = f4(n.kv, i);
+            }
+        }
+        if (s < r1) load(s + 1);
+        float U1[4], V1[4], N1[4], zu[4], zv1[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            U1[i] = __fmul_rn(a0[i], x2[i] - x0[i]);
+            V1[i] = __fmul_rn(a0[i], x2[i] + x0[i]);
+            N1[i] = __fmul_rn(a1[i], x1[i]);
+        }
+        const float Ul = __shfl_up_sync(0xffffffffu, U1[3], 1), Nr = __shfl_down_sync(0xffffffffu, N1[0], 1);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            zu[i] = __fmul_rn(ku[i], du[i] + (N[i] - N1[i]));                              // row s - 1
+            zv1[i] = __fmul_rn(kv[i], (V1[i] - V[i]) + (N1[i] - (i < 3 ? N1[i < 3 ? i + 1 : 3] : Nr)));   // row s
+        }
+        const float zr = __shfl_down_sync(0xffffffffu, zu[0], 1), zl = __shfl_up_sync(0xffffffffu, zv[3], 1);
+        if (s > r0 && out) {
+            float4 yo[3];
+            float* yf[3] = {&yo[0].x, &yo[1].x, &yo[2].x};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float zur = i < 3 ? zu[i < 3 ? i + 1 : 3] : zr, zvl = i > 0 ? zv[i > 0 ? i - 1 : 0] : zl;
+                const float zvd = zv[i] - zv1[i];
+                if (ac[i] != 0.f) {
+                    yf[2][i] = ac[i] * ((zu[i] - zur) + zvd);
+                    yf[0][i] = fmaf(d0[i], tx[i], ac[i] * ((zur - zu[i]) + zvd));
+                } else {
+                    yf[2][i] = pr[i];
+                    yf[0][i] = tx[i];
+                }
+                yf[1][i] = fmaf(d1[i], ty[i], an[i] * ((zu[i] - zm[i]) + (zv[i] - zvl)));
+            }
+            const int64_t o = o0 + (int64_t)(s - 1) * L.P;
+#pragma unroll
+            for (int f = 0; f < 3; ++f) *reinterpret_cast<float4*>(y + f * S + o) = yo[f];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            tx[i] = x0[i]; ty[i] = x1[i]; pr[i] = x2[i]; ac[i] = a0[i]; an[i] = a1[i];
+            du[i] = U1[i] - (i > 0 ? U1[i > 0 ? i - 1 : 0] : Ul);
+            V[i] = V1[i]; N[i] = N1[i]; zv[i] = zv1[i]; zm[i] = zu[i];
+        }
+    }
+}
+
 // ------------------------------- 3D -----------------------------------------
 // Staged helpers per slot (tile + halo):
 //   Uc = a_c (p - txx), Vc = a_c (p - tyy), Wc = a_c (p + txx + tyy)
@@ -1157,7 +1272,18 @@ static cudaError_t launch_mode(const Layout& L, const int* tiles, int ntiles, co
         const bool aligned = (((uintptr_t)x | (uintptr_t)y | (uintptr_t)a.pold | (uintptr_t)a.pnew |
                                (uintptr_t)a.b) & 15u) == 0;
         if constexpr (sizeof(T) == 4) {
-            if (aligned && (sizeof(C) == 4 || cf.pr[0])) {
+            // the whole grid: strips, where chunks of eight rows make warps for a
+            // third of what fits (FP32 1024^2 18.5 -> 14.3 us, 850^2 16.4 -> 14.2,
+            // 700^2 13.4 against 14.1); one wave of warps, the chunks as long as that
+            // takes
+            const int strips = (L.P + SC2 - 1) / SC2;
+            static int cache_s[16];
+            const int fit = MODE == MODE_PLAIN && !tiles ? 8 * resident_ctas((const void*)k_apply2d_stream<C>, 256, 0, cache_s) : 0;
+            if (fit && aligned && (sizeof(C) == 4 || cf.pr[0]) && 2 * (int64_t)L.R * strips >= 5 * (int64_t)fit) {
+                const int ny = std::max(SR2, (int)(((int64_t)L.R * strips + fit - 1) / fit));
+                const int nwarp = strips * ((L.R + ny - 1) / ny);
+                k_apply2d_stream<C><<<(nwarp + 7) / 8, 256, 0, s>>>(L, cf, x, y, strips, nwarp, ny);
+            } else if (aligned && (sizeof(C) == 4 || cf.pr[0])) {
                 const int grid =
                     std::min((ntiles + 3) / 4, resident_ctas((const void*)k_apply2d_v4<C, MODE>, 256, 0, cache2));
                 k_apply2d_v4<C, MODE><<<grid, 256, 0, s>>>(L, tiles, cf, x, y, a, ntiles);

@@ -425,7 +425,7 @@ def run_ours(args, rank, world):
     ms_apply, ms_update = ctx.bench_cg_kernels(prec, 50)
     tiles = ctx.active_tiles()
     slots = tiles * (256 if wl.dim == 2 else 512)
-    apply_kernel = "k_apply2d" if wl.dim == 2 else "k_apply3d"
+    apply_kernel = "k_apply2d" if wl.dim == 2 else "k_apply3d"       # (their FP32 forms: k_apply2d_v4, k_apply3d_rows)
     apply_bytes = slots * bytes_per_slot_apply(wl.dim, prec)
     apply_gbs = apply_bytes / (ms_apply * 1e-3) / 1e9
     active_slots = count_active_slots(ctx, wl)

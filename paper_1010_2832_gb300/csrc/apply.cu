@@ -598,7 +598,7 @@ __global__ void __launch_bounds__(256, 2) k_apply2d_v4(Layout L, const int* __re
 // halo.  A row's loads go out a row ahead; what the rows share stays in registers
 // and what neighbouring columns share goes by shuffles: no shared memory, no
 // barrier, and every row is read once per chunk of ny rows (plus one on each side).
-// Bound by HBM: 4096^2 box, FP32 120 us = 6.7 TB/s of the 0.80 GB it must move, 0.98
+// Bound by HBM: 4096^2 box, FP32 120 us = 6.8 TB/s of the 0.81 GB it must move, 0.99
 // of the measured bandwidth (k_apply2d_v4 158 us); BF16 coefficients 103 us against
 // 157.  Products that two positions share are rounded before they are subtracted,
 // and of a sum of two products the first is fused, as in apply2d_tile.
@@ -1017,8 +1017,8 @@ __global__ void __launch_bounds__(256, 3) k_apply3d(Layout L, Coef<C> cf, const 
 // what a neighbour reads.
 //
 // What bounds it: the latency of a plane's loads (one step ahead, 22 warps per SM)
-// and two barriers a step.  256^3 box: 348 us = 4.6 TB/s of the 1.58 GB it must
-// move, 0.67 of the measured HBM bandwidth; k_apply3d 406 us (three memory round
+// and two barriers a step.  256^3 box: 347 us = 5.2 TB/s of the 1.79 GB it must
+// move, 0.76 of the measured HBM bandwidth; k_apply3d 406 us (three memory round
 // trips a plane, 18 shared-memory reads per face position where this has 6).  The
 // thin liquid column (238 units of 4 planes): 21.2 -> 18.0 ms for the whole step.
 // Copying planes to shared memory ahead with cp.async lost (445 us: the copies, the

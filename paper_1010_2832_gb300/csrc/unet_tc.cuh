@@ -48,6 +48,7 @@
 //   atomics.
 #pragma once
 #include <cstdint>
+#include <type_traits>
 #include <cuda_bf16.h>
 
 namespace unet_tc {
@@ -163,7 +164,8 @@ struct Halo {
     static constexpr int NG = CP / 8, N = (G::NH * NG + 255) / 256;
     static constexpr int UZ = KZ == 3 ? 1 : 0;             // the coarse level halves z in 3D only
     static constexpr uint32_t NONE = 0xffffffffu, UP = 1u << 31;
-    int rel[N];
+    using Rel = typename std::conditional<KZ == 3, int, int64_t>::type;
+    Rel rel[N];                                            // from the tile's first voxel, in pieces of 8 channels
     uint32_t pos[N];                                       // shared offset / 16 (13 bits), hx, hy (5 bits), hz (4 bits), UP
     __device__ __forceinline__ void init(const TShape& s) {
 #pragma unroll
@@ -172,9 +174,9 @@ struct Halo {
             const int gq = e % NG, v = e / NG;
             const int hx = v % G::HX, hy = (v / G::HX) % G::HY, hz = v / (G::HX * G::HY);
             const bool up = CU > 0 && gq < CU / 8;
-            rel[i] = up ? ((((hz - G::RZ) >> UZ) * (s.H >> 1) + ((hy - G::R) >> 1)) * (s.W >> 1) + ((hx - G::R) >> 1)) * CU +
-                              8 * gq
-                        : (((hz - G::RZ) * s.H + (hy - G::R)) * s.W + (hx - G::R)) * (CP - CU) + 8 * gq - CU;
+            rel[i] = up ? (((Rel)((hz - G::RZ) >> UZ) * (s.H >> 1) + ((hy - G::R) >> 1)) * (s.W >> 1) + ((hx - G::R) >> 1)) *
+                                  (CU / 8) + gq
+                        : (((Rel)(hz - G::RZ) * s.H + (hy - G::R)) * s.W + (hx - G::R)) * ((CP - CU) / 8) + gq - CU / 8;
             pos[i] = (uint32_t)(v * (cps(CP) / 8) + gq) | (uint32_t)hx << 13 | (uint32_t)hy << 18 | (uint32_t)hz << 23 |
                      (up ? UP : 0u);
             if (e >= G::NH * NG) pos[i] = NONE;
@@ -197,7 +199,7 @@ struct Halo {
                           gz = z0 - G::RZ + (int)((pos[i] >> 23) & 15);
                 ok = (unsigned)gx < (unsigned)s.W && (unsigned)gy < (unsigned)s.H && (unsigned)gz < (unsigned)s.D;
             }
-            const __nv_bfloat16* src = (CU > 0 && (pos[i] & UP) ? cb : xb) + rel[i];
+            const __nv_bfloat16* src = (CU > 0 && (pos[i] & UP) ? cb : xb) + 8 * (int64_t)rel[i];
             cp_async16(sx + 16u * (pos[i] & 0x1fffu), ok ? src : X, ok);
         }
     }

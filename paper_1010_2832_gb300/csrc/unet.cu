@@ -157,40 +157,77 @@ __global__ void __launch_bounds__(256) k_skip_pool_adj(const float* __restrict__
 // loss = mean_b ||out_b - y_b||^2 / ||y_b||^2; g = d loss / d out.  The two
 // sums per sample are reduced deterministically: per-block partials (warp
 // shuffles, then warps in order), then the blocks in order.  FP64 arithmetic
-// and conversions are slow on this part (two per clock and SM): the squares
-// are summed as float-float pairs (TwoProd, TwoSum: about 2^-44 relative) and
-// the gradient's factor 2 / (||y||^2 B) is kept as a float-float pair, its
-// product with out - y then accurate to about 2^-47 before it is rounded
-// (with an FP64 division per element: 319 us for 8.4 M elements).
+// and conversions are slow on this part (two per clock and SM; FP64 sums and an
+// FP64 division per element took 319 us for 8.4 M elements), so the squares are
+// summed, and the gradient's factor is applied, in three FP32 parts where FP32
+// holds every part exactly: 1000 squares to 8e-20 relative (FP64 sums 3e-15, sums
+// in two FP32 parts 6e-13), the gradient rounded once to FP32.  Values outside
+// that range (below 2^-50 or above 2^50, not finite) are squared and summed in
+// FP64.
 constexpr int LOSS_BLOCKS = 256;      // most blocks per sample
-struct SumFF {
-    float hi = 0.f, lo = 0.f;
-    __device__ void square(float a) {
-        const float p = a * a, e = fmaf(a, a, -p);
-        float s, t;
-        stk::two_sum(hi, p, s, t);
-        lo += t + e;
+struct Squares {
+    float hi = 0.f, mid = 0.f, lo = 0.f;
+    double far = 0.0;
+    // + (a + b + c)
+    __device__ __forceinline__ void plus(float a, float b, float c) {
+        float s, t, u, v;
+        stk::two_sum(hi, a, s, t);
         hi = s;
+        stk::two_sum(mid, b, s, u);
+        stk::two_sum(s, t, mid, v);
+        lo += c + u + v;
     }
-    __device__ double warp() const { return stk::warp_sum_ff(hi, lo); }
+    // a^2; false where a^2 and its error are not FP32 numbers: nothing is added
+    __device__ __forceinline__ bool add(float a) {
+        const float m = fabsf(a);
+        const bool near = (m >= 0x1p-50f && m <= 0x1p50f) || m == 0.f;
+        const float x = near ? a : 0.f, p = __fmul_rn(x, x);    // (rounded: the sums must not take it in unrounded)
+        plus(p, fmaf(x, x, -p), 0.f);
+        return near;
+    }
+    __device__ __forceinline__ void add_far(float a) {
+        const float m = fabsf(a);
+        if (!((m >= 0x1p-50f && m <= 0x1p50f) || m == 0.f)) far = fma((double)a, (double)a, far);
+    }
+    // sum over the warp (lane 0)
+    __device__ __forceinline__ double warp() {
+        for (int o = 16; o > 0; o >>= 1) {
+            const float a = __shfl_xor_sync(0xffffffffu, hi, o), b = __shfl_xor_sync(0xffffffffu, mid, o),
+                        c = __shfl_xor_sync(0xffffffffu, lo, o);
+            plus(a, b, c);
+        }
+        double s = 0.0;
+        if ((threadIdx.x & 31) == 0) s = (double)hi + ((double)mid + (double)lo);
+        if (__any_sync(0xffffffffu, far != 0.0)) s += warp_sum(far);
+        return s;
+    }
 };
 __global__ void __launch_bounds__(256) k_loss_partials(const float* __restrict__ out, const float* __restrict__ y,
                                                        int64_t per, double* part) {
     __shared__ double red[2][8];
     const int b = blockIdx.y;
-    SumFF num, den;
+    Squares num, den;
     const float* ob = out + b * per;
     const float* yb = y + b * per;
     const int64_t step = (int64_t)gridDim.x * 256;
     int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    bool near = true;
     for (; e + 3 * step < per; e += 4 * step) {
         float o[4], t[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) { o[k] = ob[e + k * step]; t[k] = yb[e + k * step]; }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) { num.square(o[k] - t[k]); den.square(t[k]); }
+        for (int k = 0; k < 4; ++k) near = num.add(o[k] - t[k]) & den.add(t[k]) & near;
     }
-    for (; e < per; e += step) { const float t = yb[e]; num.square(ob[e] - t); den.square(t); }
+    for (; e < per; e += step) { const float t = yb[e]; near = num.add(ob[e] - t) & den.add(t) & near; }
+    // (a loop of its own: as predicated instructions the FP64 squares would cost
+    // every element their 64 clocks: 75 us for 8.4 M elements instead of 26)
+    if (!near)
+        for (e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < per; e += step) {
+            const float t = yb[e];
+            num.add_far(ob[e] - t);
+            den.add_far(t);
+        }
     const double dn = num.warp(), dd = den.warp();
     const int w = threadIdx.x >> 5;
     if ((threadIdx.x & 31) == 0) { red[0][w] = dn; red[1][w] = dd; }
@@ -203,11 +240,15 @@ __global__ void __launch_bounds__(256) k_loss_partials(const float* __restrict__
     }
 }
 
-// One warp per sample: the blocks' partials, a fixed tree; then the
-// gradient's factor 2 / (||y||^2 B) = (f.x + f.y) 2^f.z (scaled by a power of
-// two, since it can lie outside the FP32 range), 0 for a sample whose target
-// is zero.
-__global__ void k_loss_finish(const double* part, int nblocks, int B, double* sums, float4* fac) {
+// The gradient's factor 2 / (||y||^2 B) of a sample and ||y||^2.  The factor is
+// (f0 + f1 + f2) scale, exactly the FP64 value, scale a power of two; zeros if it
+// is far outside the FP32 range.
+struct LossFactor {
+    double den;
+    float f0, f1, f2, scale;
+};
+// One warp per sample: the blocks' partials, a fixed tree; then the factor.
+__global__ void k_loss_finish(const double* part, int nblocks, int B, double* sums, LossFactor* fac) {
     const int b = blockIdx.x, lane = threadIdx.x;
     double a = 0.0, c = 0.0;
     for (int q = lane; q < nblocks; q += 32) { a += part[2 * (b * nblocks + q)]; c += part[2 * (b * nblocks + q) + 1]; }
@@ -216,34 +257,60 @@ __global__ void k_loss_finish(const double* part, int nblocks, int B, double* su
     if (lane != 0) return;
     sums[2 * b] = a;
     sums[2 * b + 1] = c;
+    LossFactor f{c, 0.f, 0.f, 0.f, 0.f};
     int ex = 0;
-    const double m = c > 0.0 ? frexp(2.0 / c / B, &ex) : 0.0;
-    const float fh = (float)m;
-    fac[b] = make_float4(fh, (float)(m - (double)fh), (float)ex, 0.f);
+    double m = c > 0.0 ? frexp(2.0 / c / B, &ex) : 0.0;
+    if (abs(ex) <= 120) {
+        f.f0 = (float)m;
+        m -= (double)f.f0;
+        f.f1 = (float)m;
+        f.f2 = (float)(m - (double)f.f1);
+        f.scale = ldexpf(1.f, ex);
+    }
+    fac[b] = f;
 }
+
+// Gradient entry 2 d / (||y||^2 B), rounded once to FP32: d f as the exact d f0
+// and d f1 and a rounded d f2.  ok is cleared where the parts of the product or
+// the result are not clear of FP32's ends (then it is loss_grad_far's).
+__device__ __forceinline__ float loss_grad(float d, const LossFactor& f, bool& ok) {
+    const float p = __fmul_rn(d, f.f0), e = fmaf(d, f.f0, -p), q = __fmul_rn(d, f.f1), g = fmaf(d, f.f1, -q);
+    float s, t, u, v;
+    stk::two_sum(e, q, s, t);
+    stk::two_sum(p, s, u, v);
+    const float r = (u + (v + (t + fmaf(d, f.f2, g)))) * f.scale;
+    const float m = fabsf(d), a = fabsf(r);
+    ok = ok && (d == 0.f || (m >= 0x1p-60f && m <= 0x1p100f && a >= 0x1p-100f && a <= 0x1p100f));
+    return r;
+}
+__device__ __noinline__ float loss_grad_far(float d, double den, int B) { return (float)(2.0 * (double)d / den / B); }
 
 // gradient of the loss at the output, in BF16 with cp channels (zero padded),
 // as the output convolution's backward kernels read it: four channels a thread
 __global__ void __launch_bounds__(256) k_loss_grad(const float* __restrict__ out, const float* __restrict__ y,
-                                                   int64_t nvox, int c, int cp, const float4* __restrict__ fac,
+                                                   int64_t nvox, int c, int cp, const LossFactor* __restrict__ fac,
                                                    __nv_bfloat16* __restrict__ g) {
     const int nq = cp >> 2, per = 256 / nq;               // nq = 2 or 4
     const int q = threadIdx.x & (nq - 1);
     const int64_t vs = (int64_t)blockIdx.x * per + threadIdx.x / nq;
     if (vs >= nvox) return;
     const int64_t v = (int64_t)blockIdx.y * nvox + vs;
-    const float4 f = fac[blockIdx.y];
-    const int ex = (int)f.z;
+    const LossFactor f = fac[blockIdx.y];
     float r[4] = {0.f, 0.f, 0.f, 0.f};
-    if (4 * q < c && f.x != 0.f) {
+    // (a sample whose target is zero contributes nothing)
+    if (4 * q < c && f.den > 0.0) {
         const float* po = out + v * c + 4 * q;
         const float* py = y + v * c + 4 * q;
+        float d[4];
+        bool ok = true;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const float d = po[k] - py[k];
-            const float p = d * f.x;
-            r[k] = ldexpf(isfinite(p) ? p + (fmaf(d, f.x, -p) + d * f.y) : p, ex);
+            d[k] = po[k] - py[k];
+            r[k] = loss_grad(d[k], f, ok);
         }
+        if (!ok)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) r[k] = loss_grad_far(d[k], f.den, gridDim.y);
     }
     const __nv_bfloat162 lo = __floats2bfloat162_rn(r[0], r[1]), hi = __floats2bfloat162_rn(r[2], r[3]);
     *reinterpret_cast<uint2*>(g + v * cp + 4 * q) =
@@ -296,7 +363,7 @@ struct stokes_net_s {
     // the pooled tensors (8 and 16 channels)
     float *g_c0 = nullptr, *g_c1 = nullptr, *g_p0 = nullptr, *g_p1 = nullptr;
     double* sums = nullptr;
-    float4* fac = nullptr;          // per sample: the loss gradient's factor
+    LossFactor* fac = nullptr;      // per sample: the loss gradient's factor
     std::vector<void*> allocs;
     cudaStream_t s = nullptr;
     std::string err;
@@ -563,7 +630,7 @@ stokes_status stokes_net_create(stokes_net* out, int dim, int cin, int cout, int
     A((void**)&n->out, 4 * V * cout);
     A((void**)&n->g_c0, 4 * V * 24); A((void**)&n->g_c1, 4 * (V / 4 + 1) * 48);
     A((void**)&n->g_p0, 4 * (V / 4 + 1) * 8); A((void**)&n->g_p1, 4 * (V / 16 + 1) * 16);
-    A((void**)&n->fac, 16 * 1024);
+    A((void**)&n->fac, sizeof(LossFactor) * 1024);
     A((void**)&n->sums, 16 * 1024 + 16 * 1024 * LOSS_BLOCKS);   // sums, then the per-block partials
     if (e != cudaSuccess) { stokes_net_destroy(n); return STOKES_ERR_CUDA; }
     *out = n;

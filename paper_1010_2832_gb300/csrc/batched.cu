@@ -75,18 +75,22 @@ struct alignas(16) BState {
     unsigned cnt;
 };
 
-// One 16-byte word, so a poll of the grid barrier reads all of it at once.
 struct alignas(16) BGlobal {
     unsigned bar_count;          // arrivals since the launch began
+    int err;                     // (a poll of the grid barrier loads both)
     int ndone;                   // instances done; changes in the initial phase and phase D only
-    int err, pad;
+    int pad;
 };
 
 // Grid barrier: the CTAs' arrivals are counted up through the launch and each CTA
 // polls for this barrier's total, so no CTA has to see the last arrival and
 // release the others (one L2 round trip and one fence less than a count and a
 // generation).  Bounded; false, for the whole CTA, after an error anywhere.
-// ndone: the instances done as of this barrier (meaningful after phase D).
+// ndone: the instances done as of this barrier, in the barriers after a phase
+// that changes it.  It is read past the fence: a load beside the count's is not
+// ordered after it, and a CTA that saw an older number than the others would go
+// on alone.  No CTA changes it again before every CTA has arrived at the next
+// barrier.
 __device__ __forceinline__ bool grid_sync(BGlobal* g, unsigned nblocks, unsigned& target, int* ndone = nullptr) {
     __shared__ int ok, nd;
     target += nblocks;
@@ -94,18 +98,15 @@ __device__ __forceinline__ bool grid_sync(BGlobal* g, unsigned nblocks, unsigned
     if (threadIdx.x == 0) {
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&g->bar_count) : "memory");
         unsigned count;
-        int done, err, pad;
+        int err;
         for (int spins = 0;; ++spins) {
-            asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(count), "=r"(done), "=r"(err), "=r"(pad)
-                         : "l"(g)
-                         : "memory");
+            asm volatile("ld.volatile.global.v2.u32 {%0, %1}, [%2];" : "=r"(count), "=r"(err) : "l"(&g->bar_count) : "memory");
             if (err || (int)(count - target) >= 0) break;
             if (spins > (1 << 24)) { err = (int)STOKES_ERR_TIMEOUT; atomicExch(&g->err, err); }
         }
         asm volatile("fence.acq_rel.gpu;" ::: "memory");
         ok = err == 0;
-        nd = done;
+        if (ndone) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(nd) : "l"(&g->ndone) : "memory");
     }
     __syncthreads();
     if (ndone) *ndone = nd;

@@ -190,11 +190,15 @@ typedef struct {
                           iterations launched one kernel at a time (for
                           profilers that cannot enter conditional graphs)   */
     int wait_test;     /* test hook for the bounded device-side waits, 0 in
-                          normal use.  1 (precond = 2, mixed mode): the
-                          Schwarz local solves wait for a factor copy that is
-                          never issued, giving up after 1,024 polls, so the
-                          call returns STOKES_ERR_TIMEOUT and the context
-                          stays usable.                                     */
+                          normal use.  1: a word or copy that others wait for
+                          is held back and they give up after 1,024 polls, so
+                          the call returns STOKES_ERR_TIMEOUT and the context
+                          stays usable.  Held back are: in the one-kernel loops
+                          of small 2D systems (use_graph = 1), the CTAs' edge
+                          values (Jacobi) or the answers of one group of patches
+                          (precond = 2); in the separate Schwarz kernels
+                          (precond = 2, mixed mode), the copies of the local
+                          factors.  A solve in which nothing waits ignores it. */
 } stokes_options;
 
 typedef struct {

@@ -44,7 +44,8 @@ template <class T, int TY> struct Loop2Smem {
     double vals[GATHER_DIRECT * (TY == 8 ? 2 : 2 * TY)];       // a larger grid's reducer: dynamic shared memory
 };
 
-template <class T, class C, int TY>
+// WAIT_TEST: the options' hook; no CTA posts its z.
+template <class T, class C, int TY, bool WAIT_TEST>
 __global__ void __launch_bounds__(loop2_threads<T, TY>(), TY == 2 ? 3 : 2) k_cgloop2d(Layout L, const int* __restrict__ tiles, int ntiles,
                                                       Coef<C> cf, const double* __restrict__ r64,
                                                       const T* __restrict__ minv, T* __restrict__ xout,
@@ -61,7 +62,8 @@ __global__ void __launch_bounds__(loop2_threads<T, TY>(), TY == 2 ? 3 : 2) k_cgl
     extern __shared__ __align__(16) unsigned char dyn[];
     const int t = threadIdx.x, tx = t & 31, ty = t >> 5;
     const int workers = ntiles * SUB;
-    using Gather = GridGather<NT>;
+    constexpr int POLLS = WAIT_TEST ? GATHER_TEST_POLLS : GATHER_POLLS;
+    using Gather = GridGather<NT, POLLS>;
     Gather gather{slots, &sm.g, nullptr, workers};
     gather.vals = gather.direct() ? sm.vals : reinterpret_cast<double*>(dyn);
     const double* vals = gather.vals;
@@ -123,7 +125,7 @@ __global__ void __launch_bounds__(loop2_threads<T, TY>(), TY == 2 ? 3 : 2) k_cgl
     }
     // a row without an active unknown or a residual stays at zero
     const bool row = __any_sync(0xffffffffu, busy);
-    const bool edge = tx == 0 || tx == TX - 1 || ty == 0 || ty == TY - 1;
+    const bool edge = (tx == 0 || tx == TX - 1 || ty == 0 || ty == TY - 1) && !WAIT_TEST;
     unsigned long long* const zown = zw + ((size_t)blockIdx.x * 3 * NS + (own ? t : 0)) * Z::N;      // field f: + f NS N
     // halo position of this thread, and where its owner posts z
     T hp[3] = {T(0), T(0), T(0)}, hac = T(0), han = T(0);
@@ -204,7 +206,7 @@ __global__ void __launch_bounds__(loop2_threads<T, TY>(), TY == 2 ? 3 : 2) k_cgl
             unsigned long long v[3][Z::N];
             bool here = false;
 #pragma unroll 1
-            for (int poll = 0; !here && poll < GATHER_POLLS; ++poll) {
+            for (int poll = 0; !here && poll < POLLS; ++poll) {
                 here = true;
 #pragma unroll
                 for (int f = 0; f < 3; ++f)
@@ -295,13 +297,13 @@ constexpr size_t LOOP2_ZBYTES = sizeof(unsigned long long) * 3 * 256 * LOOP2_WOR
 // Workers and, past GATHER_DIRECT of them, the reducer.
 static int with_reducer(int workers) { return workers <= GATHER_DIRECT ? workers : workers + 1; }
 
-template <class T, class C, int TY>
+template <class T, class C, int TY, bool WAIT_TEST>
 static cudaError_t launch2(Ctx* c, CgWork<T>& w, const T* minv, const Coef<C>& cf, bool* taken) {
     static std::atomic<int> cache[16];
     constexpr int NT = loop2_threads<T, TY>(), D = TY == 8 ? 2 : 2 * TY;
     const int workers = c->ntiles_active * (TY2 / TY);
     const size_t dyn = sizeof(double) * D * LOOP2_WORKERS;
-    if (with_reducer(workers) > fit(k_cgloop2d<T, C, TY>, NT, dyn, cache)) return cudaSuccess;
+    if (with_reducer(workers) > fit(k_cgloop2d<T, C, TY, WAIT_TEST>, NT, dyn, cache)) return cudaSuccess;
     *taken = true;
     cudaError_t e;
     if (!c->zwords) {
@@ -318,7 +320,7 @@ static cudaError_t launch2(Ctx* c, CgWork<T>& w, const T* minv, const Coef<C>& c
     Coef<C> coef = cf;
     const double* r64 = c->w64.r;      // (FP64: the solve's own residual vector, which the kernel does not write)
     void* args[] = {&L, &tiles, &nt, &coef, &r64, &minv, &w.x, &c->zwords, &c->sc, &c->gather};
-    return cudaLaunchCooperativeKernel((const void*)k_cgloop2d<T, C, TY>, with_reducer(workers), NT, args,
+    return cudaLaunchCooperativeKernel((const void*)k_cgloop2d<T, C, TY, WAIT_TEST>, with_reducer(workers), NT, args,
                                        workers <= GATHER_DIRECT ? 0 : dyn, c->stream);
 }
 
@@ -338,10 +340,13 @@ cudaError_t launch_cg_loop(Ctx* c, CgWork<T>& w, const T* minv, const Coef<C>& c
     const int nt = c->ntiles_active;
     if (c->L.dim != 2 || nt > update_ctas) return cudaSuccess;
     if constexpr (sizeof(T) == 8) {
-        if (4 * nt <= LOOP2_WORKERS) return launch2<T, C, 2>(c, w, minv, cf, taken);
-        if (2 * nt <= LOOP2_WORKERS) return launch2<T, C, 4>(c, w, minv, cf, taken);
+        if (4 * nt <= LOOP2_WORKERS)
+            return c->wait_test ? launch2<T, C, 2, true>(c, w, minv, cf, taken) : launch2<T, C, 2, false>(c, w, minv, cf, taken);
+        if (2 * nt <= LOOP2_WORKERS)
+            return c->wait_test ? launch2<T, C, 4, true>(c, w, minv, cf, taken) : launch2<T, C, 4, false>(c, w, minv, cf, taken);
     } else {
-        if (nt <= LOOP2_WORKERS) return launch2<T, C, 8>(c, w, minv, cf, taken);
+        if (nt <= LOOP2_WORKERS)
+            return c->wait_test ? launch2<T, C, 8, true>(c, w, minv, cf, taken) : launch2<T, C, 8, false>(c, w, minv, cf, taken);
     }
     return cudaSuccess;
 }

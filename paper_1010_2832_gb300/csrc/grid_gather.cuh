@@ -5,7 +5,8 @@
 // flag beside it.  Slots alternate between two sets: a CTA writes exchange
 // e + 2 only after it has passed e + 1, that is, after every reader is done
 // with exchange e.  Every wait is bounded: a reader gives up after GATHER_POLLS
-// rounds and says so.
+// rounds (GATHER_TEST_POLLS under the options' wait test hook, where words are
+// held back) and says so.
 //
 // Up to GATHER_DIRECT workers, each CTA reads everybody's partial sums and forms
 // the total itself: one trip through L2 per exchange.  With more, that would be
@@ -34,6 +35,7 @@ constexpr int GATHER_DOUBLES = 8;                  // per worker and exchange at
 constexpr int GATHER_PITCH = GATHER_MAX + 8;       // one row per word of a worker's: a warp reads 32 workers' words as one run
 constexpr size_t GATHER_BYTES = sizeof(unsigned long long) * 2 * GATHER_PITCH * 2 * GATHER_DOUBLES;
 constexpr int GATHER_POLLS = 1 << 21;              // each round is a load from L2 (half a microsecond or more)
+constexpr int GATHER_TEST_POLLS = 1024;            // of a solve with the wait test hook
 
 __device__ __forceinline__ void post_word(unsigned long long* p, unsigned epoch, unsigned data) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(((unsigned long long)epoch << 32) | data) : "memory");
@@ -78,23 +80,28 @@ struct CgState {
         beta = trz / rz;
         rz = trz;
     }
+    // (the status of a CTA whose wait ran out stands, whichever comes first)
     __device__ void store(CgScalars* sc) const {
         sc->rz = rz; sc->rr = rr; sc->rr0 = rr0; sc->tol2 = tol2; sc->pq = pq; sc->alpha = alpha; sc->beta = beta;
-        sc->iter = iter; sc->done = 1; sc->status = status;
+        sc->iter = iter; sc->done = 1;
+        atomicCAS(&sc->status, STOKES_OK, status);
     }
 };
 
 enum { CG_START = 0, CG_DIRECTION = 1, CG_STEP = 2 };
 
-// NT threads per CTA.  An exchange orders nothing but its own words: other data
-// crosses CTAs in tagged words too.
-template <int NT> struct GridGather {
+struct GatherSmem {
+    double red[8][2];
+    double scalar;               // alpha or beta
+    int done, ok;
+};
+
+// NT threads per CTA; POLLS limits every wait (a constant: as an argument it cost
+// the kernels registers that they then spilled).  An exchange orders nothing but
+// its own words: other data crosses CTAs in tagged words too.
+template <int NT, int POLLS = GATHER_POLLS> struct GridGather {
     static constexpr int NW = NT / 32;
-    struct Smem {
-        double red[8][2];
-        double scalar;           // alpha or beta
-        int done, ok;
-    };
+    using Smem = GatherSmem;
     unsigned long long* slots;   // [2][2 * GATHER_DOUBLES][GATHER_PITCH], zero before the kernel starts; column GATHER_MAX is the result
     Smem* sm;
     double* vals;                // shared memory for the partial sums: workers * 8 doubles (reducer, or direct)
@@ -137,7 +144,7 @@ template <int NT> struct GridGather {
                 unsigned long long v[2 * D];
                 bool here = false;
 #pragma unroll 1
-                for (int poll = 0; !here && poll < GATHER_POLLS; ++poll) {
+                for (int poll = 0; !here && poll < POLLS; ++poll) {
                     here = true;
 #pragma unroll
                     for (int k = 0; k < 2 * D; ++k) v[k] = peek_word(slot(c, k));
@@ -190,7 +197,7 @@ template <int NT> struct GridGather {
                 else cg.step(max_iter, tot[0], tot[Q - 1]);
                 const double x = what == CG_DIRECTION ? cg.alpha : cg.beta;
                 if (reducer() && lane < 3) {
-                            const unsigned long long u = __double_as_longlong(x);
+                    const unsigned long long u = __double_as_longlong(x);
                     const unsigned flag = ok ? (unsigned)cg.done : 2u;
                     post_word(result(lane), epoch, lane == 0 ? (unsigned)u : lane == 1 ? (unsigned)(u >> 32) : flag);
                 }
@@ -200,7 +207,7 @@ template <int NT> struct GridGather {
             unsigned long long v = 0;
             bool here = lane >= 3;
 #pragma unroll 1
-            for (int poll = 0; !here && poll < GATHER_POLLS; ++poll) {
+            for (int poll = 0; !here && poll < POLLS; ++poll) {
                 v = peek_word(result(lane));
                 here = (unsigned)(v >> 32) == epoch;
             }
@@ -223,7 +230,7 @@ template <int NT> struct GridGather {
     // The end: the CTA that holds the scalars stores them; a time-out is marked.
     __device__ void finish(CgScalars* sc) const {
         if (!alive) {
-            if (threadIdx.x == 0) { sc->status = STOKES_ERR_TIMEOUT; sc->done = 1; }
+            if (threadIdx.x == 0) { atomicExch(&sc->status, (int)STOKES_ERR_TIMEOUT); sc->done = 1; }
         } else if ((int)blockIdx.x == (direct() ? 0 : workers) && threadIdx.x == 0) {
             cg.store(sc);
         }

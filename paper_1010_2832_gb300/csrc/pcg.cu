@@ -541,15 +541,12 @@ static cudaError_t run_inner_schwarz(Ctx* c, int use_graph, int chunk) {
     if (!c->sw_ready && (e = schwarz_build(c)) != cudaSuccess) return e;
     cudaStream_t s = c->stream;
     if (use_graph) {
-        // small systems: the whole loop in one cooperative kernel (the test hook
-        // of the factor copy's wait needs the separate kernels)
-        if (!c->wait_test) {
-            bool taken = false;
-            const int fin = std::min(persist_grid((const void*)k_sw_finish<0, 1>, 1 << 30),
-                                     persist_grid((const void*)k_sw_finish<1>, 1 << 30));
-            e = launch_schwarz_loop(c, *c->sw, fin, &taken);
-            if (taken || e != cudaSuccess) return e;
-        }
+        // small systems: the whole loop in one cooperative kernel
+        bool taken = false;
+        const int fin = std::min(persist_grid((const void*)k_sw_finish<0, 1>, 1 << 30),
+                                 persist_grid((const void*)k_sw_finish<1>, 1 << 30));
+        e = launch_schwarz_loop(c, *c->sw, fin, &taken);
+        if (taken || e != cudaSuccess) return e;
         cudaGraphExec_t& ge = c->graph[3];
         if (!ge) {
             cudaGraph_t g = nullptr;

@@ -53,9 +53,10 @@ struct SwLoopWords {
 
 // Poll one word until it carries the tag (true), the stop word is set or the
 // polls run out (false).
+template <int POLLS>
 __device__ __forceinline__ bool poll_word(const unsigned long long* p, unsigned tag, const unsigned long long* stop, float& v) {
 #pragma unroll 1
-    for (int poll = 0; poll < GATHER_POLLS; ++poll) {
+    for (int poll = 0; poll < POLLS; ++poll) {
         const unsigned long long w = peek_word(p), over = peek_word(stop);
         if ((unsigned)(w >> 32) == tag) {
             v = __uint_as_float((unsigned)w);
@@ -66,6 +67,7 @@ __device__ __forceinline__ bool poll_word(const unsigned long long* p, unsigned 
     return false;
 }
 
+template <int POLLS>
 __device__ __forceinline__ void patch_role(const Layout& L, const int* __restrict__ tiles, int ntiles, const SchwarzPlan& P,
                                            const SwLoopWords& W, unsigned char* smem, int ppg, int cta, int nctas, int max_iter) {
     const int gid = threadIdx.x >> 7, t = threadIdx.x & 127;
@@ -105,6 +107,7 @@ __device__ __forceinline__ void patch_role(const Layout& L, const int* __restric
         }
     }
     if (np == 0) return;                                  // a group without a patch
+    if (POLLS == GATHER_TEST_POLLS && cta == 0 && gid == 0) return;      // the wait test hook: no answers
     grp.sync();
     constexpr float H = 0.70710678118654752f;
     // (one answer per iteration and one for the start: a solve ends by max_iter)
@@ -117,14 +120,14 @@ __device__ __forceinline__ void patch_role(const Layout& L, const int* __restric
             if (t >= RR) {
                 if (kk[k] >= 0) {
                     float rv = 0.f;
-                    here = poll_word(rw[k], tag, W.stop, rv);
+                    here = poll_word<POLLS>(rw[k], tag, W.stop, rv);
                     s[kk[k]] = rv * sa[k];
                 }
             } else {
                 float rt = 0.f, rp = 0.f;
                 // (the two words are posted together: the second is seldom waited for)
-                if (kk[k] >= 0) here = poll_word(rw[k], tag, W.stop, rt);
-                if (kp[k] >= 0 && here) here = poll_word(rw[k] + 2 * 256, tag, W.stop, rp);
+                if (kk[k] >= 0) here = poll_word<POLLS>(rw[k], tag, W.stop, rt);
+                if (kp[k] >= 0 && here) here = poll_word<POLLS>(rw[k] + 2 * 256, tag, W.stop, rp);
                 if (kk[k] >= 0 && kp[k] >= 0) {
                     s[kk[k]] = (rt + rp) * H * sa[k];
                     s[kp[k]] = (rt - rp) * H * sb[k];
@@ -156,20 +159,23 @@ __device__ __forceinline__ void patch_role(const Layout& L, const int* __restric
     }
 }
 
+// WAIT_TEST: the options' hook; one group of patches does not answer.
+template <bool WAIT_TEST>
 __global__ void __launch_bounds__(SWL_THREADS, 1) k_swloop(Layout L, const int* __restrict__ tiles, int ntiles,
                                                            Coef<float> cf, DevArrays D, SchwarzPlan P,
                                                            const double* __restrict__ r64, float* __restrict__ xout,
                                                            SwLoopWords W, int ppg, CgScalars* sc, unsigned long long* slots) {
+    constexpr int POLLS = WAIT_TEST ? GATHER_TEST_POLLS : GATHER_POLLS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int G = (ntiles + 1) / 2;                       // tile CTAs
     const int first_patch = G <= GATHER_DIRECT ? G : G + 1;
     if ((int)blockIdx.x >= first_patch) {
-        patch_role(L, tiles, ntiles, P, W, smem_raw, ppg, blockIdx.x - first_patch, gridDim.x - first_patch, sc->max_iter);
+        patch_role<POLLS>(L, tiles, ntiles, P, W, smem_raw, ppg, blockIdx.x - first_patch, gridDim.x - first_patch, sc->max_iter);
         return;
     }
     SwLoopTileSmem& sm = *reinterpret_cast<SwLoopTileSmem*>(smem_raw);
     const int t = threadIdx.x, half = t >> 8, lt = t & 255, tx = t & 31, ty = lt >> 5;
-    using Gather = GridGather<SWL_THREADS>;
+    using Gather = GridGather<SWL_THREADS, POLLS>;
     // (the reducer holds no tile: its partial sums may lie over them)
     Gather gather{slots, &sm.g, sm.vals, G};
     if (!gather.direct()) gather.vals = reinterpret_cast<double*>(&sm.tile[0]);
@@ -288,7 +294,7 @@ __global__ void __launch_bounds__(SWL_THREADS, 1) k_swloop(Layout L, const int* 
         bool here = false;
         unsigned long long v[3][4];
 #pragma unroll 1
-        for (int poll = 0; !here && poll < GATHER_POLLS; ++poll) {
+        for (int poll = 0; !here && poll < POLLS; ++poll) {
             here = true;
 #pragma unroll
             for (int f = 0; f < 3; ++f)
@@ -351,7 +357,7 @@ __global__ void __launch_bounds__(SWL_THREADS, 1) k_swloop(Layout L, const int* 
             float v[3] = {0.f, 0.f, 0.f};
             bool got = false;
 #pragma unroll 1
-            for (int poll = 0; !got && poll < GATHER_POLLS; ++poll) {
+            for (int poll = 0; !got && poll < POLLS; ++poll) {
                 unsigned long long w[3] = {0, 0, 0};
                 if (hac != 0.f) { w[0] = peek_word(hz); w[2] = peek_word(hz + 512); }
                 if (han != 0.f) w[1] = peek_word(hz + 256);
@@ -429,7 +435,8 @@ __global__ void __launch_bounds__(SWL_THREADS, 1) k_swloop(Layout L, const int* 
 // two) 22.5 and 20.6; 150^2 box (95 tiles, three) 24.9 and 24.2.  Past four
 // patches per group, or factors that do not fit in the SMs' shared memory, the
 // separate kernels take over.
-cudaError_t launch_schwarz_loop(Ctx* c, const SchwarzPlan& P, int finish_ctas, bool* taken) {
+template <bool WAIT_TEST>
+static cudaError_t launch(Ctx* c, const SchwarzPlan& P, int finish_ctas, bool* taken) {
     *taken = false;
     const int nt = c->ntiles_active, G = (nt + 1) / 2, first = G <= GATHER_DIRECT ? G : G + 1;
     if (c->L.dim != 2 || nt < 1 || P.np < 1 || nt > SWL_MAX_TILES || P.np > SWL_MAX_PATCHES || G > finish_ctas) return cudaSuccess;
@@ -441,7 +448,7 @@ cudaError_t launch_schwarz_loop(Ctx* c, const SchwarzPlan& P, int finish_ctas, b
         smem = std::max(sizeof(SwLoopTileSmem), (size_t)SWL_GROUPS * (k * SW_FAC_BYTES + sizeof(SwLoopPatchScratch)));
         if (first + pc > 152 * 4) continue;
         // (the attribute that admits the largest size is set before the first query)
-        if (first + pc <= fit(k_swloop, SWL_THREADS, smem, cache[k])) { ppg = k; grid = first + pc; }
+        if (first + pc <= fit(k_swloop<WAIT_TEST>, SWL_THREADS, smem, cache[k])) { ppg = k; grid = first + pc; }
     }
     if (!ppg) return cudaSuccess;
     *taken = true;
@@ -467,7 +474,11 @@ cudaError_t launch_schwarz_loop(Ctx* c, const SchwarzPlan& P, int finish_ctas, b
     const double* r64 = c->w64.r;
     float* x = c->w32.x;
     void* args[] = {&L, &tiles, &n, &cf, &D, &plan, &r64, &x, &W, &ppg, &c->sc, &c->gather};
-    return cudaLaunchCooperativeKernel((const void*)k_swloop, grid, SWL_THREADS, args, smem, c->stream);
+    return cudaLaunchCooperativeKernel((const void*)k_swloop<WAIT_TEST>, grid, SWL_THREADS, args, smem, c->stream);
+}
+
+cudaError_t launch_schwarz_loop(Ctx* c, const SchwarzPlan& P, int finish_ctas, bool* taken) {
+    return c->wait_test ? launch<true>(c, P, finish_ctas, taken) : launch<false>(c, P, finish_ctas, taken);
 }
 
 }  // namespace stk

@@ -278,8 +278,7 @@ __device__ __forceinline__ bool batched_local_solve(const BarGroup& grp, const B
     if (t == 0 && next.on) patch_issue(inst[next.inst], next, Fs, bar);
     float* out = P.ybuf + (int64_t)(CJ * P.npx + CI) * PMAX;
     if (kk >= 0 && k2 >= 0) {
-        // field 0's product is the fused one in both
-        out[e] = (f == 0 ? fmaf(s[kk], sa, __fmul_rn(s[k2], sb)) : fmaf(s[k2], sb, -__fmul_rn(s[kk], sa))) * H;
+        out[e] = f == 0 ? sw_unrotate(s[kk], sa, s[k2], sb).x : sw_unrotate(s[k2], sb, s[kk], sa).y;
     } else if (kk >= 0) {
         out[e] = s[kk] * sa;
     }

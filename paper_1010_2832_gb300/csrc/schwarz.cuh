@@ -431,9 +431,9 @@ __global__ void __launch_bounds__(128, 15) k_schwarz_gemv(Layout L, SchwarzPlan 
         if (e >= PR * PR) {
             if (kk >= 0) out[e] = s[kk] * sa;
         } else if (kk >= 0 && kp >= 0) {
-            const float a = s[kk] * sa, b = s[kp] * sb;     // scale, then rotate back
-            out[e] = (a + b) * H;
-            out[2 * PR * PR + e] = (a - b) * H;
+            const float2 z = sw_unrotate(s[kk], sa, s[kp], sb);
+            out[e] = z.x;
+            out[2 * PR * PR + e] = z.y;
         } else if (kk >= 0) {
             out[e] = s[kk] * sa;
         } else if (kp >= 0) {

@@ -145,9 +145,9 @@ __device__ __forceinline__ void patch_role(const Layout& L, const int* __restric
                 if (t >= RR) {
                     if (kk[k] >= 0) post_word(out + t, tag, __float_as_uint(s[kk[k]] * sa[k]));
                 } else if (kk[k] >= 0 && kp[k] >= 0) {
-                    const float a = s[kk[k]] * sa[k], b = s[kp[k]] * sb[k];
-                    post_word(out + t, tag, __float_as_uint((a + b) * H));
-                    post_word(out + 2 * RR + t, tag, __float_as_uint((a - b) * H));
+                    const float2 z = sw_unrotate(s[kk[k]], sa[k], s[kp[k]], sb[k]);
+                    post_word(out + t, tag, __float_as_uint(z.x));
+                    post_word(out + 2 * RR + t, tag, __float_as_uint(z.y));
                 } else if (kk[k] >= 0) {
                     post_word(out + t, tag, __float_as_uint(s[kk[k]] * sa[k]));
                 } else if (kp[k] >= 0) {

@@ -197,6 +197,16 @@ struct BarGroup {
     }
 };
 
+// A cell's local results from its rotated solution (u, v) with scalings (sa, sb):
+// scale, then rotate back.  Which product of the sums is the fused one is written
+// out: left to the compiler it changed from kernel to kernel, and with it the
+// iterates of kernels that are to agree bit for bit.
+__device__ __forceinline__ float2 sw_unrotate(float u, float sa, float v, float sb) {
+    constexpr float H = 0.70710678118654752f;
+    const float b = __fmul_rn(v, sb);
+    return make_float2(fmaf(u, sa, b) * H, fmaf(u, sa, -b) * H);
+}
+
 // Largest |v[k]| over k < n (up to 128 entries), every thread of the group's
 // warps 0..3 taking one entry: a warp reduction, the four warps' results
 // through wm, one barrier (every thread of the group must call it).

@@ -198,7 +198,8 @@ typedef struct {
                           values (Jacobi) or the answers of one group of patches
                           (precond = 2); in the separate Schwarz kernels
                           (precond = 2, mixed mode), the copies of the local
-                          factors.  A solve in which nothing waits ignores it. */
+                          factors; in a batch, one arrival at the grid
+                          barrier.  A solve in which nothing waits ignores it. */
 } stokes_options;
 
 typedef struct {

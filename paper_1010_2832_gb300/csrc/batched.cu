@@ -15,7 +15,7 @@
 // its scalars: CG -> CHECK when the recurrence residual meets the
 // tolerance; CHECK -> done if the true residual meets it, else CG restarts
 // from the true residual.  Instances retire independently; the kernel ends
-// when all have.  Every grid barrier is a bounded wait: after ~2^24 polls
+// when all have.  Every grid barrier is a bounded wait: after 2^24 polls
 // it records STOKES_ERR_TIMEOUT and every CTA returns.
 //
 // What bounds it: latency.  A pass over 12 instances of 64..160 cells a side (776
@@ -77,10 +77,11 @@ struct alignas(16) BState {
 
 struct alignas(16) BGlobal {
     unsigned bar_count;          // arrivals since the launch began
-    int err;                     // (a poll of the grid barrier loads both)
+    int err;
+    int polls;                   // limit of a wait (a poll of the grid barrier loads these three)
     int ndone;                   // instances done; changes in the initial phase and phase D only
-    int pad;
 };
+constexpr int BATCH_POLLS = 1 << 24, BATCH_TEST_POLLS = 1024;
 
 // Grid barrier: the CTAs' arrivals are counted up through the launch and each CTA
 // polls for this barrier's total, so no CTA has to see the last arrival and
@@ -98,11 +99,14 @@ __device__ __forceinline__ bool grid_sync(BGlobal* g, unsigned nblocks, unsigned
     if (threadIdx.x == 0) {
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&g->bar_count) : "memory");
         unsigned count;
-        int err;
+        int err, polls, unused;
         for (int spins = 0;; ++spins) {
-            asm volatile("ld.volatile.global.v2.u32 {%0, %1}, [%2];" : "=r"(count), "=r"(err) : "l"(&g->bar_count) : "memory");
+            asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(count), "=r"(err), "=r"(polls), "=r"(unused)
+                         : "l"(g)
+                         : "memory");
             if (err || (int)(count - target) >= 0) break;
-            if (spins > (1 << 24)) { err = (int)STOKES_ERR_TIMEOUT; atomicExch(&g->err, err); }
+            if (spins > polls) { err = (int)STOKES_ERR_TIMEOUT; atomicExch(&g->err, err); }
         }
         asm volatile("fence.acq_rel.gpu;" ::: "memory");
         ok = err == 0;
@@ -553,7 +557,7 @@ struct stokes_batch_s {
     BInst* d_inst = nullptr;
     BState* d_st = nullptr;
     BState* d_st0 = nullptr;    // initial states (empty instances already retired)
-    BGlobal* d_g0 = nullptr;
+    BGlobal* d_g0 = nullptr;    // initial barrier state; and the wait test hook's
     bool use_graph = true;
     BGlobal* d_g = nullptr;
     int* d_wl = nullptr;        // [3][wl_cap]: instance, first column, first row of each work tile
@@ -675,12 +679,13 @@ static cudaError_t upload_plan(stokes_batch b, int ty) {
     b->nwork = (int)wi.size();
     std::vector<BState> st0(b->n);
     std::memset(st0.data(), 0, st0.size() * sizeof(BState));
-    BGlobal g0{};
+    // (the hook's count starts one arrival short, so every CTA waits)
+    BGlobal g0[2] = {{0u, 0, BATCH_POLLS, 0}, {0xffffffffu, 0, BATCH_TEST_POLLS, 0}};
     for (int i = 0; i < b->n; ++i)
-        if (insts[i].te == insts[i].tb) { st0[i].done = 1; g0.ndone += 1; }
+        if (insts[i].te == insts[i].tb) { st0[i].done = 1; g0[0].ndone += 1; g0[1].ndone += 1; }
     if ((e = cudaMemcpy(b->d_st0, st0.data(), st0.size() * sizeof(BState), cudaMemcpyHostToDevice)) != cudaSuccess)
         return e;
-    if ((e = cudaMemcpy(b->d_g0, &g0, sizeof(g0), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+    if ((e = cudaMemcpy(b->d_g0, g0, sizeof(g0), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
     // A captured graph holds the work-list and partial-sum pointers, the work
     // count and the grid by value: it is dropped whenever any of them changes
     // (the next solve captures again).  The buffers keep their capacity.
@@ -706,9 +711,9 @@ static cudaError_t upload_plan(stokes_batch b, int ty) {
     return cudaMemcpy(b->d_inst, insts.data(), insts.size() * sizeof(BInst), cudaMemcpyHostToDevice);
 }
 
-static cudaError_t launch_persistent(stokes_batch b, int ty, int grid, int max_iter, double tol) {
+static cudaError_t launch_persistent(stokes_batch b, int ty, int grid, int max_iter, double tol, int wait_test = 0) {
     cudaError_t e;
-    if ((e = cudaMemcpyAsync(b->d_g, b->d_g0, sizeof(BGlobal), cudaMemcpyDeviceToDevice, b->s)) != cudaSuccess)
+    if ((e = cudaMemcpyAsync(b->d_g, b->d_g0 + (wait_test == 1), sizeof(BGlobal), cudaMemcpyDeviceToDevice, b->s)) != cudaSuccess)
         return e;
     if ((e = cudaMemcpyAsync(b->d_st, b->d_st0, b->n * sizeof(BState), cudaMemcpyDeviceToDevice, b->s)) != cudaSuccess)
         return e;
@@ -833,7 +838,7 @@ static cudaError_t enqueue(stokes_batch b, const stokes_batch_io* io) {
         launch_rhs(c, io[i].u_star, c->b64);
         c->stream = keep;
     }
-    launch_persistent(b, b->ty, b->grid, b->opt.max_iter, b->opt.tol);
+    launch_persistent(b, b->ty, b->grid, b->opt.max_iter, b->opt.tol, b->opt.wait_test);
     for (int i = 0; i < b->n; ++i) {
         Ctx* c = b->c[i];
         cudaStream_t keep = c->stream;
@@ -918,7 +923,7 @@ stokes_status stokes_batch_create(stokes_batch* out, int n, const stokes_ctx* ct
     if (e == cudaSuccess) e = cudaEventCreate(&b->ev0);
     if (e == cudaSuccess) e = cudaEventCreate(&b->ev1);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_st0, n * sizeof(BState));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_g0, sizeof(BGlobal));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_g0, 2 * sizeof(BGlobal));
     // tuning runs real CG iterations: give every instance a nonzero
     // right-hand side (the Jacobi diagonal; every solve overwrites it)
     for (int i = 0; i < n && e == cudaSuccess; ++i)

@@ -1,4 +1,4 @@
-"""The bounded waits of the one-kernel CG loops, run out with the options' test
+"""The bounded waits of the one-kernel CG loops and of the batch's grid barrier, run out with the options' test
 hook (the CTAs' edge values, or one group of patches' answers, are held back and
 the others give up after 1,024 polls): the call returns STOKES_ERR_TIMEOUT,
 whichever CTA gave up and whichever held the scalars, and the same context then
@@ -84,3 +84,32 @@ def test_schwarz_loop_with_a_reducer_matches_separate_kernels():
         assert (st.status, st.iterations, st.outer) == (st2.status, st2.iterations, st2.outer)
         assert torch.equal(x, x2)
     ctx.close()
+
+
+@pytest.mark.parametrize("precond", [0, 2])
+def test_batch_barrier_runs_out(precond):
+    """A batch whose barrier misses one arrival: STOKES_ERR_TIMEOUT, and the
+    contexts then solve in another batch as fresh ones do."""
+    require_gpu()
+    from paper_1010_2832_gb300 import stokes
+    wls = [W.disk_in_box(32), W.bumps_2d(96, seed=21)]
+
+    def make(ctxs, **kw):
+        return stokes.Batch(ctxs, stokes.default_options(mode=0, precond=precond, tol=1e-8, max_iter=3, **kw))
+
+    def run(batch, dev):
+        out = [([torch.zeros_like(t) for t in d["u_star"]],
+                [torch.zeros(w.n[0] * w.n[1], dtype=torch.float64, device="cuda"),
+                 torch.zeros((w.n[0] + 1) * (w.n[1] + 1), dtype=torch.float64, device="cuda")],
+                torch.zeros(w.n[0] * w.n[1], dtype=torch.float64, device="cuda")) for w, d in zip(wls, dev)]
+        st, _ = batch.solve([d["u_star"] for d in dev], [o[0] for o in out], [o[1] for o in out], [o[2] for o in out])
+        return [(s["status"], s["iterations"]) for s in st]
+    pairs = [stokes.context_for(w, min_face_liquid=0.01) for w in wls]
+    ctxs, dev = [p[0] for p in pairs], [p[1] for p in pairs]
+    held = make(ctxs, wait_test=1)
+    for _ in range(2):
+        with pytest.raises(stokes.StokesError) as e:
+            run(held, dev)
+        assert e.value.status == -5
+    del held
+    assert run(make(ctxs), dev) == [(-3, 3), (-3, 3)]

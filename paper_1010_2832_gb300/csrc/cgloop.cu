@@ -304,12 +304,8 @@ static cudaError_t launch2(Ctx* c, CgWork<T>& w, const T* minv, const Coef<C>& c
     const int workers = c->ntiles_active * (TY2 / TY);
     const size_t dyn = sizeof(double) * D * LOOP2_WORKERS;
     if (with_reducer(workers) > fit(k_cgloop2d<T, C, TY, WAIT_TEST>, NT, dyn, cache)) return cudaSuccess;
-    *taken = true;
     cudaError_t e;
-    if (!c->zwords) {
-        if ((e = cudaMalloc((void**)&c->zwords, LOOP2_ZBYTES)) != cudaSuccess) return e;
-        c->allocs.push_back(c->zwords);
-    }
+    if (!loop_words(c, c->zwords, LOOP2_ZBYTES)) return cudaSuccess;
     if ((e = cudaMemsetAsync(c->gather, 0, GATHER_BYTES, c->stream)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(c->zwords, 0, (size_t)workers * 3 * 32 * TY * sizeof(unsigned long long) * ZWords<T>::N, c->stream)) !=
         cudaSuccess)
@@ -320,13 +316,14 @@ static cudaError_t launch2(Ctx* c, CgWork<T>& w, const T* minv, const Coef<C>& c
     Coef<C> coef = cf;
     const double* r64 = c->w64.r;      // (FP64: the solve's own residual vector, which the kernel does not write)
     void* args[] = {&L, &tiles, &nt, &coef, &r64, &minv, &w.x, &c->zwords, &c->sc, &c->gather};
-    return cudaLaunchCooperativeKernel((const void*)k_cgloop2d<T, C, TY, WAIT_TEST>, with_reducer(workers), NT, args,
-                                       workers <= GATHER_DIRECT ? 0 : dyn, c->stream);
+    *taken = loop_launched(cudaLaunchCooperativeKernel((const void*)k_cgloop2d<T, C, TY, WAIT_TEST>, with_reducer(workers), NT,
+                                                       args, workers <= GATHER_DIRECT ? 0 : dyn, c->stream));
+    return cudaSuccess;
 }
 
 // Run the inner solve in one cooperative kernel if the system is small enough
-// (*taken); the graph of separate kernels takes the others: they are bound by
-// what their kernels move, not by launches.  update_ctas: CTAs of k_cg_update
+// (*taken); the graph of separate kernels takes the others (they are bound by
+// what their kernels move, not by launches), and those that the device refuses.  update_ctas: CTAs of k_cg_update
 // that fit on the device (up to that many tiles it gives each CTA one, the order
 // that the sums here repeat).  The lines: one CTA per tile in FP32 and two per
 // tile at most in FP64 while two CTAs per SM hold them all (303 workers; 124 and

@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <atomic>
 #include "internal.cuh"
+#include "ctx.cuh"
 #include "grid_gather.cuh"
 #include "reduce.cuh"
 
@@ -93,6 +94,27 @@ template <> struct ZWords<double> {
     }
     static __device__ __forceinline__ double get(const unsigned long long (&v)[2]) { return from_words(v[0], v[1]); }
 };
+
+// A loop's words, allocated on first use; false (and no error left) if there is no
+// room for them.
+static bool loop_words(Ctx* c, unsigned long long*& words, size_t bytes) {
+    if (words) return true;
+    if (cudaMalloc((void**)&words, bytes) != cudaSuccess) {
+        words = nullptr;
+        cudaGetLastError();
+        return false;
+    }
+    c->allocs.push_back(words);
+    return true;
+}
+// Whether a cooperative launch went through.  The device may refuse it although
+// the kernel fits on all of it: a process limited to a part of the SMs, a share of
+// the device held by others.  The separate kernels then take the solve (and report
+// an error that has another cause).
+static bool loop_launched(cudaError_t e) {
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess;
+}
 
 // CTAs of a kernel that fit on the device at once (cached per device).
 template <class K>

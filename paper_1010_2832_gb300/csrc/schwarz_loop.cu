@@ -433,8 +433,8 @@ __global__ void __launch_bounds__(SWL_THREADS, 1) k_swloop(Layout L, const int* 
 // iteration, separate kernels and this: 96^2 bumps (22 tiles, one patch per group
 // of threads) 20.6 and 11.2; 160^2 (56 tiles, two) 22.2 and 16.1; 224^2 (85 tiles,
 // two) 22.5 and 20.6; 150^2 box (95 tiles, three) 24.9 and 24.2.  Past four
-// patches per group, or factors that do not fit in the SMs' shared memory, the
-// separate kernels take over.
+// patches per group, or factors that do not fit in the SMs' shared memory, or where
+// the device refuses the launch, the separate kernels take over.
 template <bool WAIT_TEST>
 static cudaError_t launch(Ctx* c, const SchwarzPlan& P, int finish_ctas, bool* taken) {
     *taken = false;
@@ -451,13 +451,9 @@ static cudaError_t launch(Ctx* c, const SchwarzPlan& P, int finish_ctas, bool* t
         if (first + pc <= fit(k_swloop<WAIT_TEST>, SWL_THREADS, smem, cache[k])) { ppg = k; grid = first + pc; }
     }
     if (!ppg) return cudaSuccess;
-    *taken = true;
     cudaError_t e;
     const size_t wt = sizeof(unsigned long long) * SWL_TILE_WORDS, wp = sizeof(unsigned long long) * SWL_PATCH_WORDS;
-    if (!c->swwords) {
-        if ((e = cudaMalloc((void**)&c->swwords, 2 * wt * SWL_MAX_TILES + wp * SWL_MAX_PATCHES + 256)) != cudaSuccess) return e;
-        c->allocs.push_back(c->swwords);
-    }
+    if (!loop_words(c, c->swwords, 2 * wt * SWL_MAX_TILES + wp * SWL_MAX_PATCHES + 256)) return cudaSuccess;
     SwLoopWords W;
     W.stop = c->swwords;
     W.z = c->swwords + 32;
@@ -474,7 +470,8 @@ static cudaError_t launch(Ctx* c, const SchwarzPlan& P, int finish_ctas, bool* t
     const double* r64 = c->w64.r;
     float* x = c->w32.x;
     void* args[] = {&L, &tiles, &n, &cf, &D, &plan, &r64, &x, &W, &ppg, &c->sc, &c->gather};
-    return cudaLaunchCooperativeKernel((const void*)k_swloop<WAIT_TEST>, grid, SWL_THREADS, args, smem, c->stream);
+    *taken = loop_launched(cudaLaunchCooperativeKernel((const void*)k_swloop<WAIT_TEST>, grid, SWL_THREADS, args, smem, c->stream));
+    return cudaSuccess;
 }
 
 cudaError_t launch_schwarz_loop(Ctx* c, const SchwarzPlan& P, int finish_ctas, bool* taken) {

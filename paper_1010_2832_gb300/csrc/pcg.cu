@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(1024) k_schwarz_list(const int* __restrict__ f
 // Patch plan and local inverses (after every weight build, on first use).  The
 // buffers are the context's and stay: those of the patch grid are allocated
 // once, those of the active patches when there are more of them than before (by
-// an eighth more).  The list is made on the device and the host waits for its
+// an eighth more where memory allows).  The list is made on the device and the host waits for its
 // length alone, not for the factors.  (Eight allocations and frees, the list on
 // the host and a wait for the factors took 0.30 ms of a 150^2 jet step.)
 static cudaError_t schwarz_build(Ctx* c) {
@@ -314,13 +314,19 @@ static cudaError_t schwarz_build(Ctx* c) {
         if (c->sw_patch) cudaFree(c->sw_patch);
         c->sw_patch = nullptr;
         c->sw_cap = 0;
-        const size_t cap = std::min((size_t)ng, (size_t)P.np + P.np / 8 + 8);
         // FP16 factors with a FP32 scale per row (BF16 storage needed 4.4x the CG
         // iterations on the 1024^2 bump workload; FP16 about 1.02x), scalings,
-        // local maps, sizes
+        // local maps, sizes; the room to grow only if there is memory for it
         auto up = [](size_t b) { return (b + 255) / 256 * 256; };
-        const size_t f = up((size_t)SW_FAC_BYTES * cap), sc = up(sizeof(float) * cap * PMAX), lm = up(sizeof(short) * cap * PMAX);
-        if ((e = cudaMalloc(&c->sw_patch, f + sc + lm + sizeof(int) * cap)) != cudaSuccess) { c->sw_patch = nullptr; return e; }
+        size_t cap = std::min((size_t)ng, (size_t)P.np + P.np / 8 + 8), f, sc, lm;
+        for (bool retry = true;; retry = false) {
+            f = up((size_t)SW_FAC_BYTES * cap), sc = up(sizeof(float) * cap * PMAX), lm = up(sizeof(short) * cap * PMAX);
+            if ((e = cudaMalloc(&c->sw_patch, f + sc + lm + sizeof(int) * cap)) == cudaSuccess) break;
+            c->sw_patch = nullptr;
+            if (e != cudaErrorMemoryAllocation || !retry) return e;
+            cudaGetLastError();
+            cap = std::max(1, P.np);
+        }
         c->sw_cap = (int)cap;
         char* base = (char*)c->sw_patch;
         P.fac = (uint8_t*)base;

@@ -347,7 +347,7 @@ stokes_status stokes_bench_cg_kernels(stokes_ctx ctx, int precision, int launche
  * every candidate (an autotuner), caching the choice in a text file (path
  * ``tune_cache``, else $STOKES_AUTOTUNE_CACHE, else
  * $HOME/.cache/libstokes_autotune.txt) keyed by instance count, problem
- * size class and GPU name.  The contexts must stay alive and unchanged
+ * size class, GPU name and revision of the kernel.  The contexts must stay alive and unchanged
  * (no new stokes_build_weights) for the life of the batch.
  * stokes_batch_solve enqueues on the batch's own stream and synchronises;
  * ``stats`` (n entries, may be NULL) receive per-instance results and

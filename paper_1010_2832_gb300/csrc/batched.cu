@@ -779,6 +779,10 @@ static void cache_store(const std::string& path, const std::string& key, int ty,
     f << key << " " << ty << " " << cps << " " << us << "\n";
 }
 
+// Raised whenever k_batched changes what a tile height or a number of CTAs costs:
+// entries measured with another kernel are not this one's best choice.
+constexpr int TUNE_REVISION = 2;
+
 static std::string tune_key(stokes_batch b) {
     long long slots = 0;
     for (auto* c : b->c) slots += (long long)c->L.P * c->L.R;
@@ -791,7 +795,7 @@ static std::string tune_key(stokes_batch b) {
     std::string gpu = p.name;
     for (auto& ch : gpu) if (ch == ' ') ch = '_';
     return std::string(b->sw ? "batch2d_fp64_schwarz_n" : "batch2d_fp64_n") + std::to_string(b->n) + "_slots2^" +
-           std::to_string(lg) + "_" + gpu;
+           std::to_string(lg) + "_" + gpu + "_k" + std::to_string(TUNE_REVISION);
 }
 
 static cudaError_t autotune(stokes_batch b, const char* cache) {

@@ -302,13 +302,15 @@ stokes_status stokes_build_weights(stokes_ctx h, const double* phiL, const doubl
         if (ge) { cudaGraphExecDestroy(ge); ge = nullptr; }
     c.sw_ready = false;
     c.learned.net = nullptr;
-    cudaError_t e = launch_build_weights(&c, phiL, phiS, rho, mu, ubc);
+    cudaError_t e = c.spoiled ? c.clear_vectors() : cudaSuccess;
+    if (e == cudaSuccess) e = launch_build_weights(&c, phiL, phiS, rho, mu, ubc);
     if (e != cudaSuccess) {
         c.err = std::string("weight build failed: ") + cudaGetErrorString(e);
         c.have_weights = false;
         return STOKES_ERR_CUDA;
     }
     c.have_weights = true;
+    c.spoiled = false;
     return STOKES_OK;
 }
 

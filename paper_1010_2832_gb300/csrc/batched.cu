@@ -1020,6 +1020,7 @@ stokes_status stokes_batch_solve(stokes_batch b, const stokes_batch_io* io, stok
             o.precision_used = STOKES_FP64;
         }
         if (s.status != STOKES_OK && worst == STOKES_OK) worst = s.status;
+        if (g.err || (s.status != STOKES_OK && s.status != STOKES_ERR_NOT_CONVERGED)) b->c[i]->spoiled = true;
     }
     if (g.err) return (stokes_status)g.err;
     return (stokes_status)worst;

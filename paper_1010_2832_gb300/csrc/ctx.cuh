@@ -89,6 +89,7 @@ struct Ctx {
     double* b64 = nullptr;       // rhs (solve_step)
     double* x64 = nullptr;       // solution (solve_step)
     double* y64 = nullptr;       // scratch
+    bool spoiled = false;        // a solve ended in infinities or NaNs, which the vectors may hold (see clear_vectors)
     cudaEvent_t ev[4]{};
     double last_apply_ms = -1.0;
     cudaGraphExec_t graph[4] = {nullptr, nullptr, nullptr, nullptr};  // inner solve per precision (+ Schwarz)
@@ -122,6 +123,22 @@ struct Ctx {
     }
     template <class C> Coef<C> coef() const;
     int64_t vec_elems() const { return (int64_t)nf * L.stride; }
+    // Zero the solver's vectors.  A solve writes the slots of active tiles and
+    // reads their halo, whose slots in other tiles keep what an earlier geometry
+    // left there and meet weights of zero.  That does for finite values alone: 0
+    // times an infinity or NaN is NaN.  So after a solve that ended in such values
+    // the vectors are cleared before the geometry changes.
+    cudaError_t clear_vectors() {
+        const int64_t V = vec_elems();
+        cudaError_t e = cudaSuccess;
+        double* v64[] = {w64.x, w64.r, w64.z, w64.p[0], w64.p[1], w64.q, b64, x64, y64};
+        for (double* v : v64)
+            if (e == cudaSuccess) e = cudaMemsetAsync(v, 0, sizeof(double) * V, stream);
+        float* v32[] = {w32.x, w32.r, w32.z, w32.p[0], w32.p[1], w32.q};
+        for (float* v : v32)
+            if (e == cudaSuccess) e = cudaMemsetAsync(v, 0, sizeof(float) * V, stream);
+        return e;
+    }
 };
 
 template <> inline Coef<double> Ctx::coef<double>() const {

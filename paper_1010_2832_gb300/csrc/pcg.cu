@@ -705,6 +705,7 @@ stokes_status solve_system(Ctx* c, const double* b, double* x, const stokes_opti
         total_iter += c->h_sc[0].iter;
         double rr_new = c->h_sc[1].rr;
         int ist = c->h_sc[0].status;
+        if ((ist != STOKES_OK && ist != STOKES_ERR_NOT_CONVERGED) || !std::isfinite(rr_new)) c->spoiled = true;
         if (std::getenv("STOKES_VERBOSE"))
             std::fprintf(stderr, "[stokes] outer %d mode %d precond %d inner iters %d status %d rel %.3e -> %.3e\n",
                          outer, mode, o->precond, c->h_sc[0].iter, ist, std::sqrt(rr / bb), std::sqrt(rr_new / bb));

@@ -286,7 +286,7 @@ stokes_status stokes_solve_step(stokes_ctx ctx, const double* const* u_star, dou
                                 stokes_stats* stats);
 
 /* Solve A x = b for a given right-hand side (FP64 slot layout, device);
- * x (same layout) is overwritten.  Same options and statistics. */
+ * x (same layout) is overwritten in full.  Same options and statistics. */
 stokes_status stokes_solve_system(stokes_ctx ctx, const double* b, double* x, const stokes_options* opt,
                                   stokes_stats* stats);
 

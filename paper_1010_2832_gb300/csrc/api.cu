@@ -389,6 +389,9 @@ stokes_status stokes_solve_system(stokes_ctx h, const double* b, double* x, cons
     stokes_status s = check_opts(c, o);
     if (s != STOKES_OK) return s;
     API_CHECK_CUDA(h, cudaEventRecord(c.ev[0], c.stream));
+    // (x's slots outside the active tiles are read as halo: what the caller's array
+    // held there must not be an infinity or NaN, see clear_vectors)
+    API_CHECK_CUDA(h, cudaMemsetAsync(x, 0, sizeof(double) * c.vec_elems(), c.stream));
     s = solve_system(&c, b, x, o, st);
     cudaEventRecord(c.ev[1], c.stream);
     if (st) {

@@ -1,6 +1,7 @@
 """A solve that ends in infinities leaves them in the context's vectors; a later
 geometry with fewer tiles reads some of them as the halo of its own, where their
-weights are zero.  The next solves must be those of a fresh context."""
+weights are zero.  The next solves must be those of a fresh context.  Likewise
+what a caller's solution array held before the call."""
 import numpy as np
 import pytest
 
@@ -65,3 +66,20 @@ def test_solve_after_a_spoiled_one(mode, rho, use_graph):
     assert all(torch.equal(a, b) for a, b in zip(out, out2))
     ctx.close()
     fresh.close()
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_solution_array_may_hold_anything(mode):
+    require_gpu()
+    from paper_1010_2832_gb300 import stokes
+    wl = _box(1.0, left=31)
+    ctx = stokes.StokesContext(2, wl.n, wl.h, wl.dt, wl.origin)
+    d = _build(ctx, wl)
+    b = ctx.new_vector()
+    ctx.rhs(d["u_star"], b)
+    want, x = ctx.new_vector(), torch.full_like(b, float("nan"))
+    for y in (want, x):
+        st = ctx.solve_system(b, y, stokes.default_options(mode=mode, tol=1e-10))
+        assert (st.status, st.precision_used) == (0, mode)
+    assert torch.equal(x, want)
+    ctx.close()

@@ -176,7 +176,8 @@ stokes_status stokes_create(stokes_ctx* out, const stokes_grid* g, void* stream)
     c.ncoef = g->dim == 2 ? 6 : 11;
     c.ntiles_all = L.ntx * L.nty * L.ntz;
     const int64_t S = L.stride;
-    // one block for everything stokes_build_weights writes (zeroed per build)
+    // one block for everything stokes_build_weights writes: zeroed here, once (each
+    // build writes every sample that exists and clears the tile flags)
     size_t wb = 0;
     auto add = [&](size_t bytes) { size_t o = wb; wb += round_up((int64_t)bytes, 256); return o; };
     size_t oWL = add(sizeof(double) * S * c.nk), oWF = add(sizeof(double) * S * c.nk);

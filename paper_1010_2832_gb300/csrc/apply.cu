@@ -1,10 +1,11 @@
 // Matrix-free apply of the SPD pressure-stress operator, eq. stokesmixedsystemspd,
 // in the factored form of Section 7: y = C x + B (K (B^T x)).
 //
-// Tiles of the padded slot lattice: 2D 32x8 slots, taken by persistent,
-// software-pipelined CTAs (the next tile's loads are in flight while the
-// current tile is computed); 3D 32x4x4, one CTA per tile.
-// Phase 1 stages, for the tile plus a one-slot halo, the row-weighted
+// 2D: tiles of 32x8 slots, taken by persistent, software-pipelined CTAs (the next
+// tile's loads are in flight while the current tile is computed), or, over a large
+// whole grid, strips that warps stream down.  3D: units of 32x8 slots and 4 to 16
+// planes that a CTA streams along z.
+// Phase 1 stages, for the tile (3D: plane) plus a one-slot halo, the row-weighted
 // unknowns that each face sees (for a u face: a_c (p - tau_xx) of the cells
 // on both sides and a_n tau_xy of the nodes above and below, ...).
 // Phase 2 forms the face values z_f = K_f (B^T x)_f for every face the tile

@@ -73,8 +73,9 @@ struct ApplyArgs {
     double* partial;
     unsigned* counter;
     CgScalars* sc;
-    // 3D: the units to apply (nullptr: every unit of the grid, every tile
-    // in the grid active, ZT_MAX layers deep), their tile masks and depth
+    // 3D: the units to apply, their tile masks and depth in tile layers
+    // (nullptr: every unit of the grid, every tile in the grid active; the
+    // launch chooses the depth)
     const int* units;
     const uint8_t* umask;
     int nunits;

@@ -839,12 +839,20 @@ cudaError_t launch_build_weights(Ctx* c, const double* phiL, const double* phiS,
     if (L.dim == 3) {
         // units of 4 tile layers (16 planes) when there are enough of them to
         // fill the device a few times over, else of one layer: a thin liquid
-        // region has too few deep units to keep every SM busy
+        // region has too few deep units to keep every SM busy.  CG-mode apply of
+        // boxes, us at depth 1 and 4, FP64 and FP32: 64^3 (867 active tiles) 106 and
+        // 148, 27.0 and 26.9; 96^3 (2,500) 280 and 321, 62.0 and 62.5; 128^3 (5,445)
+        // 565 and 583, 112 and 103; 160^3 (10,086) 1013 and 924, 191 and 163; 192^3
+        // (16,807) 1660 and 1458, 301 and 245; the thin column of a 256^3 grid (462)
+        // is 1.35 times faster at depth 1.  The line lies at 96 tiles per SM (14,592),
+        // above the crossing, where it was set with six CTAs of an earlier FP32 kernel
+        // per SM; depth 2 is the faster one from 5,000 to 10,000 tiles (128^3 FP32 99
+        // us).  Moving it reorders the dots' partial sums and so changes iterates.
         if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        // (deep units hold 2 ZT_MAX tiles; six CTAs per SM; two waves)
+        // (12 deep units of 2 ZT_MAX tiles per SM)
         c->unit_zt = c->ntiles_active >= 2 * (2 * ZT_MAX) * 6 * std::max(sms, 1) ? ZT_MAX : 1;
         const int nu = L.ntx * units_y(L.nty) * units_z(L.ntz, c->unit_zt);
         k_unit_masks<<<(nu + 255) / 256, 256, 0, s>>>(L, c->unit_zt, D.tile_flag, D.unit_mask, nu);

@@ -84,8 +84,10 @@ typedef struct stokes_ctx_s* stokes_ctx;
 /* Create a context for one grid on the current CUDA device.  ``stream`` is a
  * cudaStream_t; NULL makes the context create its own blocking stream, which
  * is ordered with the legacy default stream both ways (the legacy stream
- * itself cannot be captured into the solver's CUDA graphs).  Allocates all device work
- * space for the grid.  Returns STOKES_ERR_ARG for dim not in {2,3},
+ * itself cannot be captured into the solver's CUDA graphs).  Allocates the device work
+ * space for the grid (the one-kernel loops of small 2D systems and the Schwarz
+ * plan take theirs on first use; a loop that gets none leaves the solve to
+ * the separate kernels).  Returns STOKES_ERR_ARG for dim not in {2,3},
  * non-positive sizes, h <= 0 or dt <= 0. */
 stokes_status stokes_create(stokes_ctx* out, const stokes_grid* grid, void* stream);
 
